@@ -161,6 +161,14 @@ __device__ __forceinline__ float pair_bound(float ra, float sa, float rb, float 
     return __fadd_rn(__fadd_rn(__fmul_rn(K, q), __fmul_rn(kKappa, __fadd_rn(sa, sb))), 2.0f * kTau);
 }
 
+// One pair bound for all hits of a station, from the largest r and the largest
+// |s_x|, |s_y| (an l1 is at most twice that): pair_bound with R_a = R_b = r and
+// S_a = S_b = 2 smax, where the root is sqrt(2) r (rounded up here) at any
+// magnitude.
+__device__ __forceinline__ float station_pair_bound(float r, float smax, float K) {
+    return __fadd_rn(__fadd_rn(__fmul_rn(K, __fmul_rn(1.41421366f, r)), __fmul_rn(4.0f * kKappa, smax)), 2.0f * kTau);
+}
+
 // May hits i and j belong to one passing triplet?  (never false for such a
 // pair when bb >= fl(b_i + b_j), or bb >= the pair bound of their layers)
 __device__ __forceinline__ bool pair_ok(float sxi, float syi, float sxj, float syj, float bb) {
