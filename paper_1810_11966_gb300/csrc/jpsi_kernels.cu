@@ -64,7 +64,6 @@ namespace basek {
 constexpr bool kStream = JPSI_STREAM != 0;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kQCap = 128;                // pair queue entries per warp
-constexpr int kWalkCells = 512;           // tiles of at most this many cells per layer walk pair windows per lane
 
 // warp path: size limits of an event on it
 constexpr int kTCap = 64;                 // passing trigger triplets per event on the medium tile (CHAIN)
@@ -146,6 +145,8 @@ struct BlockSmem {
     float2 P[B::HCAP];
     uint16_t idx[B::HCAP];
     uint32_t queue[B::WARPS][kQCap];
+    uint32_t pend_pair[B::WARPS][32];        // triples that wait for their fit: i | j << 16 (tile positions)
+    uint16_t pend_k[B::WARPS][32];           //   and k
     alignas(4) uint16_t bst[3 * B::NC + 1];  // cell starts (cell counts while a layer is staged)
     LayerMeta meta[3];
     int32_t off[3 * kMaxStations + 1];
@@ -228,18 +229,6 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
         if (lane >= d) v += o;
     }
     return v;
-}
-
-// Index of the lane whose exclusive prefix `excl` is the last one <= it
-// (excl non-decreasing over the lanes): binary lifting over shuffles.
-__device__ __forceinline__ int owner_lane(int excl, int it) {
-    int o = 0;
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-        const int ex = __shfl_sync(kFull, excl, o + s);
-        o += (ex <= it) ? s : 0;
-    }
-    return o;
 }
 
 // Pulls the hit lines [h0, h1) of x, y, z into L2 (addresses stay inside the
@@ -490,55 +479,13 @@ struct TSink {
     float2* tt = nullptr;               // free-streaming windows: their (min t, max t) beside T
 };
 
-// Items of up to 32 lanes laid end to end: lane i owns items [excl, excl +
-// n0 + n1), the first n0 at tile positions a.., the others at a2.. (runs of
-// win_runs).  An item's owner is found by owner_lane over excl.
-struct Runs {
-    int excl, total;    // this lane's first item; items of the warp
-    int sa, split, sb;  // item it of this lane sits at (it < split ? sa : sb) + it
-    bool two;           // some lane has a second run (warp-uniform)
-};
-
-template <int NY>
-__device__ __forceinline__ Runs runs_scan(int a, int n0, int a2, int n1, int lane) {
-    Runs r;
-    const int len = n0 + n1;
-    const int incl = warp_incl_scan(len, lane);
-    r.total = __shfl_sync(kFull, incl, 31);
-    r.excl = incl - len;
-    r.sa = a - r.excl;
-    r.split = r.excl + n0;
-    r.sb = a2 - r.split;
-    r.two = NY > 1 && __any_sync(kFull, n1 > 0);  // one-row tiles never have a second run
-    return r;
-}
-
-// Tile position of item `it`, owned by lane o (all lanes call it).
-template <int NY>
-__device__ __forceinline__ int runs_pos(const Runs& r, int o, int it) {
-    const int pa = __shfl_sync(kFull, r.sa, o) + it;
-    if (NY == 1 || !r.two) return pa;
-    const int sp = __shfl_sync(kFull, r.split, o), pb = __shfl_sync(kFull, r.sb, o) + it;
-    return it < sp ? pa : pb;
-}
-
-// Position of the k-th (0-based) set bit of m (binary lifting over the
-// counts of lower bits; k < popc(m)).
-__device__ __forceinline__ int nth_set_bit(unsigned m, int k) {
-    int pos = 0;
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1)
-        if (__popc(m & ((1u << (pos + s)) - 1u)) <= k) pos += s;
-    return pos;
-}
-
-// Triples that passed both pair tests and wait for their exact fit (block
-// paths): lane l < m holds one, as tile positions i | j << 16 and k.  The
-// fits (and the global loads of their hits) then run 32 at a time.
+// Triples that passed all pair tests and wait for their exact fit (block
+// paths): the warp's m entries in shared memory.  The fits (and the global
+// loads of their hits) then run 32 at a time.
 struct Pending {
-    uint32_t pair = 0;
-    int k = 0;
-    int m = 0;
+    uint32_t* pair;
+    uint16_t* k;
+    int m;
 };
 
 // P1 on the triples of the lanes with `has` (layer-local hits ii, jj, kk of
@@ -630,55 +577,55 @@ __device__ __forceinline__ void fit_tile(const Job& j, const TV& t, int lane, co
 }
 
 // Drains a pair queue: every (i, j) against the L2 hits in the meet of both
-// cell windows.  The (pair, k) items of up to 32 pairs are spread evenly over
-// the lanes (a warp prefix sum over the window sizes; each lane finds the
-// pair owning its item by binary lifting).  Items that pass both pair tests
-// join the pending triples of `pd`, so that the global loads of the fits run
-// for 32 triples at a time.
+// cell windows.  Each lane walks the window of its own pair (both runs), as long
+// as the longest of the 32: pairs of one queue come from neighbouring hits, so
+// their windows are alike, and a step costs a load, two pair tests and a vote.
+// Triples that pass all pair tests join the pending ones, which are fitted 32 at
+// a time.  (Spreading the items of all windows evenly over the lanes cost an
+// owner search of five shuffles a step and two searches for the n-th set bit per
+// vote: 2 000 dense events 12.06 -> 11.40 ms without them, the block tiles of
+// 100 000 free-streaming collisions 2.21 -> 2.00 ms, of a 55 000-event log-normal
+// timeslice 0.946 -> 0.913 ms.)
 template <bool EMIT, class TV>
 __device__ void drain(const Job& j, const TV& t, const uint32_t* queue, int lane, const Cuts& c, int qn,
                       TSink& ts, int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag, int& count,
                       Pending& pd) {
     const float B02 = layer_pair_bound(t, 0, 2, c.K), B12 = layer_pair_bound(t, 1, 2, c.K);
+    const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll 1
     for (int q0 = 0; q0 < qn; q0 += 32) {
-        const int q = q0 + lane;
-        uint32_t en = 0;
+        const uint32_t en = queue[min(q0 + lane, qn - 1)];
+        const float2 Pi = t.P[en & 0xffffu], Pj = t.P[en >> 16];
         int a = 0, m0 = 0, a2 = 0, m1 = 0;
-        if (q < qn) {
-            en = queue[q];
-            const float2 Pi = t.P[en & 0xffffu], Pj = t.P[en >> 16];
+        if (q0 + lane < qn) {
             const Win w = win_meet(cell_window(t, 2, Pi.x, Pi.y, B02, B02), cell_window(t, 2, Pj.x, Pj.y, B12, B12));
             win_runs(t, 2, w, a, m0, a2, m1);
         }
-        const Runs rr = runs_scan<TV::NY>(a, m0, a2, m1, lane);
-        const int total = rr.total;
-        for (int it0 = 0; it0 < total; it0 += 32) {
-            const int it = it0 + lane;
-            const int o = owner_lane(rr.excl, it);
-            const uint32_t eo = __shfl_sync(kFull, en, o);
-            const int ko = runs_pos<TV::NY>(rr, o, it);
-            const bool in = it < total;
-            const int ko_c = in ? ko : (int)(eo >> 16);
-            const float2 Pi = t.P[eo & 0xffffu], Pj = t.P[eo >> 16], Pk = t.P[ko_c];
-            const bool cand = in & pair_ok(Pi.x, Pi.y, Pk.x, Pk.y, B02) & pair_ok(Pj.x, Pj.y, Pk.x, Pk.y, B12);
-            unsigned mask = __ballot_sync(kFull, cand);
-            while (mask) {  // warp-uniform: candidates of rank r go to lane pd.m + r
-                const int np = __popc(mask), take = min(np, 32 - pd.m);
-                const int r = lane - pd.m;
-                const int src = nth_set_bit(mask, min(max(r, 0), np - 1));
-                const uint32_t vp = __shfl_sync(kFull, eo, src);
-                const int vk = __shfl_sync(kFull, ko_c, src);
-                if (r >= 0 && r < take) {
-                    pd.pair = vp;
-                    pd.k = vk;
+        const int len = m0 + m1, nmax = __reduce_max_sync(kFull, len);
+#pragma unroll 1
+        for (int k = 0; k < nmax; ++k) {
+            const int pk = k < m0 ? a + k : a2 + (k - m0);
+            const float2 Pk = t.P[k < len ? pk : 0];
+            const bool cand = (k < len) & pair_ok(Pi.x, Pi.y, Pk.x, Pk.y, B02) & pair_ok(Pj.x, Pj.y, Pk.x, Pk.y, B12);
+            const unsigned mask = __ballot_sync(kFull, cand);
+            if (!mask) continue;
+            const int at = pd.m + __popc(mask & lt);
+            if (cand && at < 32) {
+                pd.pair[at] = en;
+                pd.k[at] = (uint16_t)pk;
+            }
+            pd.m += __popc(mask);
+            if (pd.m >= 32) {
+                __syncwarp();
+                const uint32_t pe = pd.pair[lane];
+                fit_tile<EMIT>(j, t, lane, c, true, (int)(pe & 0xffffu), (int)(pe >> 16), pd.k[lane], ts, rows, limit,
+                               unit, sh_rank, tag, count);
+                __syncwarp();
+                if (cand && at >= 32) {
+                    pd.pair[at - 32] = en;
+                    pd.k[at - 32] = (uint16_t)pk;
                 }
-                pd.m += take;
-                mask = take == np ? 0u : mask & ~((1u << nth_set_bit(mask, take)) - 1u);
-                if (pd.m == 32) {
-                    fit_tile<EMIT>(j, t, lane, c, true, (int)(pd.pair & 0xffffu), (int)(pd.pair >> 16), pd.k, ts, rows,
-                                   limit, unit, sh_rank, tag, count);
-                    pd.m = 0;
-                }
+                pd.m -= 32;
             }
         }
     }
@@ -690,9 +637,11 @@ template <bool EMIT, class TV>
 __device__ __forceinline__ void flush_pending(const Job& j, const TV& t, int lane, const Cuts& c, TSink& ts,
                                               int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag,
                                               int& count, Pending& pd) {
-    if (pd.m > 0)
-        fit_tile<EMIT>(j, t, lane, c, lane < pd.m, (int)(pd.pair & 0xffffu), (int)(pd.pair >> 16), pd.k, ts, rows,
-                       limit, unit, sh_rank, tag, count);
+    if (pd.m > 0) {
+        const uint32_t pe = pd.pair[min(lane, pd.m - 1)];
+        fit_tile<EMIT>(j, t, lane, c, lane < pd.m, (int)(pe & 0xffffu), (int)(pe >> 16), pd.k[min(lane, pd.m - 1)], ts,
+                       rows, limit, unit, sh_rank, tag, count);
+    }
     pd.m = 0;
 }
 
@@ -711,12 +660,10 @@ struct RoadItems {
 
 // All passing triplets of the staged station (Sec. 3.2 steps 1-2) found by
 // this warp: rounds of 32 L0 hits, taken from a counter that the warps of the
-// block share.  On the medium tile each lane walks its own hit's L1 window; on
-// the block tile each hit's window (its runs of cells) is spread over the
-// lanes so every lane tests one candidate pair per step.  Pairs that may
-// belong to a passing triplet are queued and drained against L2.
+// block share.  Each lane walks its own hit's L1 window.  Pairs that may belong to
+// a passing triplet are queued and drained against L2.
 template <bool EMIT, class TV>
-__device__ int enum_station(const Job& j, const TV& t, uint32_t* queue, int lane, const Cuts& c,
+__device__ int enum_station(const Job& j, const TV& t, uint32_t* queue, Pending pd, int lane, const Cuts& c,
                             TSink& ts, int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag, int* sh_next,
                             const RoadItems* rd) {
     const int n0 = t.meta[0].nlive, n1 = t.meta[1].nlive, n2 = t.meta[2].nlive;
@@ -725,7 +672,6 @@ __device__ int enum_station(const Job& j, const TV& t, uint32_t* queue, int lane
     const int p0 = t.meta[0].pbase;
     const float B01 = layer_pair_bound(t, 0, 1, c.K);
     int qn = 0, count = 0;
-    Pending pd;
     // each warp takes the next round from the block-shared counter; items past
     // the rounds are trigger slopes to search for (CHAIN)
     auto next_round = [&]() {
@@ -733,7 +679,8 @@ __device__ int enum_station(const Job& j, const TV& t, uint32_t* queue, int lane
         if (lane == 0) g = atomicAdd(sh_next, 1);
         return 32 * __shfl_sync(kFull, g, 0);
     };
-    int i0 = next_round();
+    auto next_work = [&]() {
+        int i0 = next_round();
         while (rd && i0 >= n0 && (i0 >> 5) - n_rounds < rd->n) {
             const int ti = (i0 >> 5) - n_rounds;
             if (rd->alive[ti]) {
@@ -743,71 +690,36 @@ __device__ int enum_station(const Job& j, const TV& t, uint32_t* queue, int lane
             }
             i0 = next_round();
         }
-    for (; i0 < n0;) {
+        return i0;
+    };
+    for (;;) {
+        const int i0 = next_work();
+        if (i0 >= n0) break;
         const bool has = i0 + lane < n0;
         const float2 Pi = t.P[p0 + (has ? i0 + lane : 0)];
         int a = 0, m0 = 0, a2 = 0, m1 = 0;
         if (has) win_runs(t, 1, cell_window(t, 1, Pi.x, Pi.y, B01, B01), a, m0, a2, m1);
-        if constexpr (TV::NC <= kWalkCells) {
-            // medium tile: each lane walks its own hit's window (both runs),
-            // as long as the warp's longest.  The 32 L0 hits of a round are
-            // neighbours in the cell order, so their windows are alike, and a
-            // step costs a load, the test and a vote instead of the balanced
-            // step's owner search: 3 % less kernel time on the log-normal
-            // timeslices.  The block tile's wider windows keep balanced steps.
-            const int len = m0 + m1;
-            const int nmax = __reduce_max_sync(kFull, len);
-            for (int k = 0; k < nmax; ++k) {
-                const bool in = k < len;
-                const int pj = k < m0 ? a + k : a2 + (k - m0);
-                const float2 Pj = t.P[in ? pj : p0];
-                const bool pass = in & pair_ok(Pi.x, Pi.y, Pj.x, Pj.y, B01);
-                const unsigned mask = __ballot_sync(kFull, pass);
-                if (mask) {
-                    const int qi = qn + __popc(mask & lanemask_lt());
-                    if (pass && JPSI_IN(j.ctrl, qi < kQCap)) queue[qi] = (uint32_t)(p0 + i0 + lane) | ((uint32_t)pj << 16);
-                    qn += __popc(mask);
-                    if (qn > kQCap - 32) {
-                        __syncwarp();
-                        drain<EMIT>(j, t, queue, lane, c, qn, ts, rows, limit, unit, sh_rank, tag, count, pd);
-                        qn = 0;
-                    }
-                }
+        // each lane walks its own hit's window (both runs), as long as the
+        // warp's longest: the 32 L0 hits of a round are neighbours in the cell
+        // order, so their windows are alike
+        const int len = m0 + m1;
+        const int nmax = __reduce_max_sync(kFull, len);
+#pragma unroll 1
+        for (int k = 0; k < nmax; ++k) {
+            const bool in = k < len;
+            const int pj = k < m0 ? a + k : a2 + (k - m0);
+            const float2 Pj = t.P[in ? pj : p0];
+            const bool pass = in & pair_ok(Pi.x, Pi.y, Pj.x, Pj.y, B01);
+            const unsigned mask = __ballot_sync(kFull, pass);
+            if (!mask) continue;
+            const int qi = qn + __popc(mask & lanemask_lt());
+            if (pass && JPSI_IN(j.ctrl, qi < kQCap)) queue[qi] = (uint32_t)(p0 + i0 + lane) | ((uint32_t)pj << 16);
+            qn += __popc(mask);
+            if (qn > kQCap - 32) {
+                __syncwarp();
+                drain<EMIT>(j, t, queue, lane, c, qn, ts, rows, limit, unit, sh_rank, tag, count, pd);
+                qn = 0;
             }
-        } else {
-            const Runs rr = runs_scan<TV::NY>(a, m0, a2, m1, lane);
-            const int total = rr.total;
-            for (int it0 = 0; it0 < total; it0 += 32) {
-                const int it = it0 + lane;
-                const int o = owner_lane(rr.excl, it);
-                const int pj = runs_pos<TV::NY>(rr, o, it);
-                const bool in = it < total;
-                const float2 Po = t.P[p0 + i0 + o];
-                const float2 Pj = t.P[in ? pj : p0];
-                const bool pass = in & pair_ok(Po.x, Po.y, Pj.x, Pj.y, B01);
-                const unsigned mask = __ballot_sync(kFull, pass);
-                if (mask) {
-                    const int qi = qn + __popc(mask & lanemask_lt());
-                    if (pass && JPSI_IN(j.ctrl, qi < kQCap))
-                        queue[qi] = (uint32_t)(p0 + i0 + o) | ((uint32_t)pj << 16);
-                    qn += __popc(mask);
-                    if (qn > kQCap - 32) {
-                        __syncwarp();
-                        drain<EMIT>(j, t, queue, lane, c, qn, ts, rows, limit, unit, sh_rank, tag, count, pd);
-                        qn = 0;
-                    }
-                }
-            }
-        }
-        i0 = next_round();
-        while (rd && i0 >= n0 && (i0 >> 5) - n_rounds < rd->n) {
-            const int ti = (i0 >> 5) - n_rounds;
-            if (rd->alive[ti]) {
-                const float2 m = rd->T[ti];
-                const bool found = road_warp(j, t, c, m.x, m.y, rd->Tt ? rd->Tt[ti] : make_float2(0.f, 0.f), lane);
-                if (lane == 0 && !found) rd->alive[ti] = 0;
-            }
-            i0 = next_round();
         }
     }
     __syncwarp();
@@ -1750,7 +1662,8 @@ __device__ bool heavy_unit(const Job& j, BlockSmem<B>& sm, const Cuts& c, int gi
     // enumeration rounds (both only read the staged tile)
     const bool empty = sm.meta[0].nlive == 0 || sm.meta[1].nlive == 0 || sm.meta[2].nlive == 0;
     const RoadItems rd{T, alive, EMIT || empty ? 0 : nT, Tt};
-    enum_station<EMIT>(j, TV{sm.P, sm.idx, sm.bst, sm.meta}, sm.queue[wp], lane, c, ts, rows,
+    enum_station<EMIT>(j, TV{sm.P, sm.idx, sm.bst, sm.meta}, sm.queue[wp],
+                       Pending{sm.pend_pair[wp], sm.pend_k[wp], 0}, lane, c, ts, rows,
                        cnt_expected, u, &sm.s_rank, B::CLS, &sm.s_next, &rd);
     __syncthreads();
     cnt = sm.s_rank;
