@@ -68,6 +68,11 @@ struct Graph {
     std::vector<cudaKernelNodeParams> params;
 };
 
+// The captured phases.  A timed run takes light, rest and scatter one by one, with
+// events between them; any other run has the count (light + rest), and the scatter
+// with it when it records triplets, in one graph and waits once.
+enum Phase { kPhLight, kPhRest, kPhEmit, kPhScatter, kPhCount, kPhCountRows, kPhases };
+
 // Per-run state: job, control block, graphs.  The serving loop owns one per
 // slot; plain runs use the context's own.
 struct RunState {
@@ -79,7 +84,7 @@ struct RunState {
     DevBuf dpair, tlist_ijk, tpool_ijk;  // distinct_hits
     DevBuf zfill, ztab;  // per-hit z filled from a batch's z_layer table; the table on the device
     int64_t tscr_want = (int64_t)1 << 22;  // entries; grows after an overflow
-    Graph g_light, g_rest, g_emit, g_scatter;
+    Graph graphs[kPhases];    // captured when first needed
     int g_cfg_id = -1;
     bool g_stream = false;  // the graphs hold the free-streaming kernels
     cudaEvent_t ev[9] = {};  // timing marks: light start/end, rest end, emit start/end; window build and rows
@@ -115,10 +120,11 @@ struct Launchers {
     decltype(&basek::launch_plain_light) plain_light;
     decltype(&basek::launch_plain_rest) plain_rest;
     decltype(&basek::launch_plain_emit) plain_emit;
+    decltype(&basek::useful_blocks) useful_blocks;
 };
 const Launchers kEventL{false, basek::launch_light_count, basek::launch_count_rest, basek::launch_emit_phase,
                         basek::launch_scatter, basek::launch_plain_light, basek::launch_plain_rest,
-                        basek::launch_plain_emit};
+                        basek::launch_plain_emit, basek::useful_blocks};
 // Time inputs of a run over free-streaming windows (device pointers).
 struct StreamJob {
     const float* t;   // [window-batch hits]
@@ -128,7 +134,7 @@ struct StreamJob {
 
 const Launchers kStreamL{true, streamk::launch_light_count, streamk::launch_count_rest, streamk::launch_emit_phase,
                          streamk::launch_scatter, streamk::launch_plain_light, streamk::launch_plain_rest,
-                         streamk::launch_plain_emit};
+                         streamk::launch_plain_emit, streamk::useful_blocks};
 
 }  // namespace
 
@@ -335,7 +341,10 @@ jpsi_status prepare(jpsi_ctx* c, RunState& rs, const jpsi_batch* b, jpsi_outputs
     j.cx = c->cx;
     j.cy = c->cy;
     j.K = c->K;
-    j.grab = c->tune.light_grab;
+    // events per grab: one until every resident warp has two grabs (64 events,
+    // two warps' worth of the default grab, took twice an event's time)
+    const int64_t warps = (int64_t)c->batch_cfg.light_blocks * c->batch_cfg.light_wpb;
+    j.grab = (int32_t)std::max<int64_t>(1, std::min<int64_t>(c->tune.light_grab, ne / (2 * std::max<int64_t>(warps, 1))));
     j.cap_small = c->tune.small_layer_cap;
     j.cap_medium = c->tune.medium_layer_cap;
     j.host_hits = host_hits ? 1 : 0;
@@ -393,11 +402,10 @@ jpsi_status state_init(jpsi_ctx* c, RunState& rs) {
 }
 
 void destroy_graphs(RunState& rs) {
-    Graph* gs[] = {&rs.g_light, &rs.g_rest, &rs.g_emit, &rs.g_scatter};
-    for (Graph* g : gs) {
-        if (g->exec) cudaGraphExecDestroy(g->exec);
-        if (g->g) cudaGraphDestroy(g->g);
-        *g = Graph{};
+    for (Graph& g : rs.graphs) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        if (g.g) cudaGraphDestroy(g.g);
+        g = Graph{};
     }
 }
 
@@ -436,57 +444,69 @@ void state_free(jpsi_ctx* c, RunState& rs) {
     release(c, rs.tscr);
 }
 
-// Captures the count and emit phases of the batched form into graphs (with
-// the current job; graph_launch writes each run's job into their nodes).
-jpsi_status capture_graphs(jpsi_ctx* c, RunState& rs, const Launchers& L = kEventL) {
-    if (rs.g_light.exec && rs.g_cfg_id == c->cfg_id && rs.g_stream == L.stream) return JPSI_OK;
+// The graph of a phase of the batched form, captured if it is not there yet for
+// the context's launch shape and these kernels (with the current job; phase_launch
+// writes each run's job into its nodes).
+jpsi_status phase_graph(jpsi_ctx* c, RunState& rs, Phase phase, const Launchers& L, Graph** out) {
+    Graph& G = rs.graphs[phase];
+    *out = &G;
+    const bool same = rs.g_cfg_id == c->cfg_id && rs.g_stream == L.stream;
+    if (G.exec && same) return JPSI_OK;
     std::lock_guard<std::mutex> cap_lock(c->cap_mu);
-    destroy_graphs(rs);
-    for (int phase = 0; phase < 4; ++phase) {
-        Graph& G = phase == 0 ? rs.g_light : phase == 1 ? rs.g_rest : phase == 2 ? rs.g_emit : rs.g_scatter;
-        cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) return cuda_fail(c, e, "graph capture");
-        cudaError_t le = phase == 0   ? L.light_count(rs.job, 0, c->batch_cfg, true, c->cap_stream)
-                         : phase == 1 ? L.count_rest(rs.job, c->batch_cfg, c->cap_stream)
-                         : phase == 2 ? L.emit_phase(rs.job, 0, c->batch_cfg, true, c->cap_stream)
-                                      : L.scatter(rs.job, c->batch_cfg, c->cap_stream);
-        e = cudaStreamEndCapture(c->cap_stream, &G.g);
-        if (le != cudaSuccess) return cuda_fail(c, le, "graph capture launch");
-        if (e != cudaSuccess) return cuda_fail(c, e, "graph end capture");
-        size_t n = 0;
-        if ((e = cudaGraphGetNodes(G.g, nullptr, &n)) != cudaSuccess) return cuda_fail(c, e, "graph nodes");
-        std::vector<cudaGraphNode_t> all(n);
-        if (n && (e = cudaGraphGetNodes(G.g, all.data(), &n)) != cudaSuccess) return cuda_fail(c, e, "graph nodes");
-        for (cudaGraphNode_t node : all) {
-            cudaGraphNodeType t;
-            if ((e = cudaGraphNodeGetType(node, &t)) != cudaSuccess) return cuda_fail(c, e, "graph node type");
-            if (t != cudaGraphNodeTypeKernel) continue;
-            cudaKernelNodeParams kp{};
-            if ((e = cudaGraphKernelNodeGetParams(node, &kp)) != cudaSuccess) return cuda_fail(c, e, "graph node");
-            G.nodes.push_back(node);
-            G.params.push_back(kp);
-        }
-        if ((e = cudaGraphInstantiate(&G.exec, G.g, 0)) != cudaSuccess) return cuda_fail(c, e, "graph instantiate");
-    }
+    if (!same) destroy_graphs(rs);
     rs.g_cfg_id = c->cfg_id;
     rs.g_stream = L.stream;
+    cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return cuda_fail(c, e, "graph capture");
+    cudaError_t le = cudaSuccess;
+    if (phase == kPhLight || phase == kPhCount || phase == kPhCountRows)
+        le = L.light_count(rs.job, 0, c->batch_cfg, true, c->cap_stream);
+    if (le == cudaSuccess && (phase == kPhRest || phase == kPhCount || phase == kPhCountRows))
+        le = L.count_rest(rs.job, c->batch_cfg, c->cap_stream);
+    if (le == cudaSuccess && (phase == kPhScatter || phase == kPhCountRows))
+        le = L.scatter(rs.job, c->batch_cfg, c->cap_stream);
+    if (le == cudaSuccess && phase == kPhEmit) le = L.emit_phase(rs.job, 0, c->batch_cfg, true, c->cap_stream);
+    e = cudaStreamEndCapture(c->cap_stream, &G.g);
+    if (le != cudaSuccess) return cuda_fail(c, le, "graph capture launch");
+    if (e != cudaSuccess) return cuda_fail(c, e, "graph end capture");
+    size_t n = 0;
+    if ((e = cudaGraphGetNodes(G.g, nullptr, &n)) != cudaSuccess) return cuda_fail(c, e, "graph nodes");
+    std::vector<cudaGraphNode_t> all(n);
+    if (n && (e = cudaGraphGetNodes(G.g, all.data(), &n)) != cudaSuccess) return cuda_fail(c, e, "graph nodes");
+    G.nodes.clear();
+    G.params.clear();
+    for (cudaGraphNode_t node : all) {
+        cudaGraphNodeType t;
+        if ((e = cudaGraphNodeGetType(node, &t)) != cudaSuccess) return cuda_fail(c, e, "graph node type");
+        if (t != cudaGraphNodeTypeKernel) continue;
+        cudaKernelNodeParams kp{};
+        if ((e = cudaGraphKernelNodeGetParams(node, &kp)) != cudaSuccess) return cuda_fail(c, e, "graph node");
+        G.nodes.push_back(node);
+        G.params.push_back(kp);
+    }
+    if ((e = cudaGraphInstantiate(&G.exec, G.g, 0)) != cudaSuccess) return cuda_fail(c, e, "graph instantiate");
     return JPSI_OK;
 }
 
-// Replays a captured phase for `job`: every kernel node of the graph takes
-// the job as its only parameter (warp kernels in their persistent form).
-cudaError_t graph_launch(Graph& G, const Job& job, cudaStream_t st) {
-    Job j = job;
+// Replays a captured phase for the current job: every kernel node of the graph
+// takes the job as its only parameter (warp kernels in their persistent form).
+jpsi_status phase_launch(jpsi_ctx* c, RunState& rs, Phase phase, const Launchers& L, cudaStream_t st) {
+    Graph* G = nullptr;
+    const jpsi_status s = phase_graph(c, rs, phase, L, &G);
+    if (s != JPSI_OK) return s;
+    Job j = rs.job;
     j.persistent = 1;
     void* args[] = {&j};
-    for (size_t i = 0; i < G.nodes.size(); ++i) {
-        cudaKernelNodeParams kp = G.params[i];
+    cudaError_t e = cudaSuccess;
+    for (size_t i = 0; i < G->nodes.size() && e == cudaSuccess; ++i) {
+        cudaKernelNodeParams kp = G->params[i];
         kp.kernelParams = args;
         kp.extra = nullptr;
-        const cudaError_t e = cudaGraphExecKernelNodeSetParams(G.exec, G.nodes[i], &kp);
-        if (e != cudaSuccess) return e;
+        kp.gridDim.x = L.useful_blocks(kp.func, j, kp.gridDim.x);
+        e = cudaGraphExecKernelNodeSetParams(G->exec, G->nodes[i], &kp);
     }
-    return cudaGraphLaunch(G.exec, st);
+    if (e == cudaSuccess) e = cudaGraphLaunch(G->exec, st);
+    return e == cudaSuccess ? JPSI_OK : cuda_fail(c, e, "graph launch");
 }
 
 // Accumulates per-phase device times of a finished run (events already complete).
@@ -533,14 +553,27 @@ jpsi_status run_device(jpsi_ctx* c, RunState& rs, const jpsi_batch* b, jpsi_outp
     if (c->p.distinct_hits && ne > 0 && (e = cudaMemsetAsync(rs.dpair.p, 0, (size_t)ne, st)) != cudaSuccess)
         return cuda_fail(c, e, "flag reset");
     const bool timing = c->timing.load();
-    if (batched && (s = capture_graphs(c, rs, L)) != JPSI_OK) return s;
-    if (timing) cudaEventRecord(rs.ev[0], st);
-    e = batched ? graph_launch(rs.g_light, rs.job, st) : L.plain_light(rs.job, c->plain_cfg, st);
-    if (e != cudaSuccess) return cuda_fail(c, e, "light count");
-    if (timing) cudaEventRecord(rs.ev[1], st);
-    e = batched ? graph_launch(rs.g_rest, rs.job, st) : L.plain_rest(rs.job, c->plain_cfg, st);
-    if (e != cudaSuccess) return cuda_fail(c, e, "count rest");
-    if (timing) cudaEventRecord(rs.ev[2], st);
+    // A batched run with room for the triplet record scatters it behind the
+    // count, without waiting for the count in between (k_scatter does nothing
+    // unless the record and the caller's buffer hold every triplet).
+    const bool joined = batched && !timing, rows_joined = joined && o->triplets && rs.job.tscr;
+    if (joined) {
+        if ((s = phase_launch(c, rs, rows_joined ? kPhCountRows : kPhCount, L, st)) != JPSI_OK) return s;
+    } else {
+        if (timing) cudaEventRecord(rs.ev[0], st);
+        if (batched) {
+            if ((s = phase_launch(c, rs, kPhLight, L, st)) != JPSI_OK) return s;
+        } else if ((e = L.plain_light(rs.job, c->plain_cfg, st)) != cudaSuccess) {
+            return cuda_fail(c, e, "light count");
+        }
+        if (timing) cudaEventRecord(rs.ev[1], st);
+        if (batched) {
+            if ((s = phase_launch(c, rs, kPhRest, L, st)) != JPSI_OK) return s;
+        } else if ((e = L.plain_rest(rs.job, c->plain_cfg, st)) != cudaSuccess) {
+            return cuda_fail(c, e, "count rest");
+        }
+        if (timing) cudaEventRecord(rs.ev[2], st);
+    }
     int launches = batched ? kLaunchesLight + kLaunchesRest : kLaunchesPlainLight + kLaunchesPlainRest;
     if ((e = cudaMemcpyAsync(rs.h_ctrl, rs.d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
         return cuda_fail(c, e, "ctrl readback");
@@ -567,12 +600,14 @@ jpsi_status run_device(jpsi_ctx* c, RunState& rs, const jpsi_batch* b, jpsi_outp
                            ctl.scratch_n <= (unsigned long long)rs.job.tscr_cap;
     if (!scattered && rs.job.tscr && !(ctl.status & kStNoScratch))
         rs.tscr_want = std::max<int64_t>(rs.tscr_want, (int64_t)(ctl.scratch_n + ctl.scratch_n / 4));
+    if (scattered && rows_joined) return JPSI_OK;  // the rows are there
     if (timing) cudaEventRecord(rs.ev[3], st);
-    if (scattered)
-        e = batched ? graph_launch(rs.g_scatter, rs.job, st) : L.scatter(rs.job, c->plain_cfg, st);
-    else
-        e = batched ? graph_launch(rs.g_emit, rs.job, st) : L.plain_emit(rs.job, c->plain_cfg, st);
-    if (e != cudaSuccess) return cuda_fail(c, e, "emit");
+    if (batched) {
+        if ((s = phase_launch(c, rs, scattered ? kPhScatter : kPhEmit, L, st)) != JPSI_OK) return s;
+    } else {
+        e = scattered ? L.scatter(rs.job, c->plain_cfg, st) : L.plain_emit(rs.job, c->plain_cfg, st);
+        if (e != cudaSuccess) return cuda_fail(c, e, "emit");
+    }
     if (timing) cudaEventRecord(rs.ev[4], st);
     launches += scattered ? kLaunchesScatter : batched ? kLaunchesEmit : kLaunchesPlainEmit;
     if ((e = cudaMemcpyAsync(rs.h_ctrl, rs.d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
@@ -1346,7 +1381,10 @@ jpsi_status jpsi_serve_start(jpsi_ctx* c, int n_slots, int64_t slot_events, int6
             (s = ensure(c, sl->rs.block_sums, (size_t)((nu + 4095) / 4096 + 1) * 8, "slot scan")))
             break;
         // graphs are captured with the context's launch shape
-        if ((s = capture_graphs(c, sl->rs)) != JPSI_OK) break;
+        Graph* g = nullptr;
+        if ((s = phase_graph(c, sl->rs, kPhCount, kEventL, &g)) != JPSI_OK ||
+            (s = phase_graph(c, sl->rs, kPhCountRows, kEventL, &g)) != JPSI_OK)
+            break;
         c->free_slots.push_back(i);
     }
     if (s != JPSI_OK) {

@@ -154,6 +154,8 @@ struct LaunchCfg {
 //   launch_plain_*: the one-launch form (no lists, queues or graphs): the
 //     static warp grid (1), then the static block grid and the tail (1 + 4);
 //     its emit fallback is the two static grids again (2).
+//   useful_blocks: how many blocks of a kernel of the counting phase can have
+//     work.
 //   launch_expand_z: per-hit z of events [ev0, ev1) from a per-layer table.
 #define JPSI_DECLARE_LAUNCHERS                                                                                  \
     cudaError_t launch_light_count(const Job& j, int64_t n_events, const LaunchCfg& lc, bool persistent,    \
@@ -175,6 +177,7 @@ struct LaunchCfg {
     int heavy_max_blocks_per_sm();                                                                            \
     int medium_max_blocks_per_sm();                                                                           \
     size_t heavy_smem_bytes();                                                                                \
+    unsigned useful_blocks(const void* kernel, const Job& j, unsigned full);                                  \
     const void* light_count_kernel_ptr();
 
 namespace basek {

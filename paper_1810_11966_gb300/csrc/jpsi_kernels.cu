@@ -159,6 +159,17 @@ struct BlockSmem {
 };
 using HeavySmem = BlockSmem<HeavyCfg>;
 
+// The kernels of a run are launched one behind the other with programmatic
+// serialization.  chain_wait, the first statement of each: its work starts when the
+// kernel before it is complete.  chain_next: the next kernel's blocks may be set
+// up (and wait) once all blocks of this grid have come here or ended; small
+// kernels say so at once, the persistent ones when they run out of work (earlier,
+// the waiting blocks would keep shared memory from other streams' kernels:
+// twelve timeslices over three serving slots 3.01 -> 3.17 ms).  Both are no-ops in
+// a launch without the attribute.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 __device__ __forceinline__ unsigned lanemask_lt() {
     unsigned m;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
@@ -1541,6 +1552,7 @@ __device__ __forceinline__ void light_event(const Job& j, WarpTile& w, int lane,
 template <bool EMIT>
 __global__ void __maxnreg__(72) k_light(const __grid_constant__ Job j) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     WarpTile& w = reinterpret_cast<WarpTile*>(smem_raw)[wi];
     const Cuts c{j.cx, j.cy, j.K};
@@ -1560,6 +1572,7 @@ __global__ void __maxnreg__(72) k_light(const __grid_constant__ Job j) {
 #pragma unroll 1
         for (int k = k0; k < k1; ++k) light_event<EMIT>(j, w, lane, c, j.ev_begin + k);
     }
+    chain_next();
 }
 
 // ------------------------------------------------------ block-tile path
@@ -1862,6 +1875,7 @@ __device__ void medium_event(const Job& j, MediumSmem& ms, const Cuts& c, int64_
 template <bool EMIT>
 __global__ void __launch_bounds__(MedBCfg::THREADS, 14) k_medium(const __grid_constant__ Job j) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     MediumSmem& ms = *reinterpret_cast<MediumSmem*>(smem_raw);
     const Cuts c{j.cx, j.cy, j.K};
     const int n_med = *(volatile int32_t*)&j.ctrl->n_medium, m0 = *(volatile int32_t*)&j.ctrl->m_begin;
@@ -1876,6 +1890,7 @@ __global__ void __launch_bounds__(MedBCfg::THREADS, 14) k_medium(const __grid_co
         if (!EMIT || j.ev_class[e] == kClsMedium) medium_event<EMIT>(j, ms, c, e);
         __syncthreads();
     }
+    chain_next();
 }
 
 // Orders the block-tile list by decreasing event size (hits, in kSortBins
@@ -1891,6 +1906,8 @@ __global__ void __launch_bounds__(1024) k_sort_heavy(const __grid_constant__ Job
     __shared__ uint8_t cls[kSortCap];
     __shared__ int start[kSortBins];
     __shared__ int s_max;
+    chain_next();
+    chain_wait();
     const int h0 = *(volatile int32_t*)&j.ctrl->h_begin;
     const int n = *(volatile int32_t*)&j.ctrl->n_heavy - h0;
     int32_t* list = j.hlist + h0;
@@ -1952,6 +1969,7 @@ __global__ void __launch_bounds__(1024) k_sort_heavy(const __grid_constant__ Job
 // Counting pass: persistent blocks take block-tile events from the list.
 __global__ void __launch_bounds__(kHThreads, 3) k_heavy(const __grid_constant__ Job j) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     HeavySmem& sm = *reinterpret_cast<HeavySmem*>(smem_raw);
     const Cuts c{j.cx, j.cy, j.K};
     const int n_heavy = *(volatile int32_t*)&j.ctrl->n_heavy, h0 = *(volatile int32_t*)&j.ctrl->h_begin;
@@ -1964,6 +1982,7 @@ __global__ void __launch_bounds__(kHThreads, 3) k_heavy(const __grid_constant__ 
         heavy_event(j, sm, c, gi, j.hlist[gi]);
         __syncthreads();
     }
+    chain_next();
 }
 
 // One block per (event, station) unit of the block-tile path.  Counting pass
@@ -1972,6 +1991,7 @@ __global__ void __launch_bounds__(kHThreads, 3) k_heavy(const __grid_constant__ 
 template <bool EMIT>
 __global__ void __launch_bounds__(kHThreads, 3) k_heavy_units(const __grid_constant__ Job j) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     HeavySmem& sm = *reinterpret_cast<HeavySmem*>(smem_raw);
     const int S = j.S;
     if (!EMIT && (j.mode != 1 || S < 2)) return;
@@ -2020,11 +2040,14 @@ __global__ void __launch_bounds__(kHThreads, 3) k_heavy_units(const __grid_const
                          kStream ? reinterpret_cast<const float2*>(j.tpool_ijk) + hx : nullptr);
         __syncthreads();
     }
+    chain_next();
 }
 
 // CHAIN track counts of the events whose stations ran on separate blocks:
 // the trigger slopes still alive after every station (one warp per event).
 __global__ void k_heavy_final(const __grid_constant__ Job j) {
+    chain_next();
+    chain_wait();
     if (j.mode != 1 || j.S < 2) return;
     const int n_heavy = *(volatile int32_t*)&j.ctrl->n_heavy, h0 = *(volatile int32_t*)&j.ctrl->h_begin;
     const int lane = threadIdx.x & 31;
@@ -2284,6 +2307,7 @@ __global__ void __launch_bounds__(kGenThreads) k_generic(const __grid_constant__
     __shared__ int32_t soff[3 * kMaxStations + 1];
     __shared__ int s_gi, s_count, s_cand, s_bad;
     __shared__ unsigned long long s_pool;
+    chain_wait();
     const int n_gen = *(volatile int32_t*)&j.ctrl->n_generic, g0 = *(volatile int32_t*)&j.ctrl->g_begin;
     for (;;) {
         if (threadIdx.x == 0) s_gi = g0 + (int)atomicAdd(&j.ctrl->work[EMIT ? 7 : 3], 1ull);
@@ -2295,6 +2319,7 @@ __global__ void __launch_bounds__(kGenThreads) k_generic(const __grid_constant__
             generic_event<EMIT>(j, e, GenShared{soff, &s_count, &s_cand, &s_bad, &s_pool});
         __syncthreads();
     }
+    chain_next();
 }
 
 // ------------------------------------------------- one-launch form, blocks
@@ -2430,6 +2455,7 @@ __device__ bool plain_block_event(const Job& j, PlainSmem& ps, int64_t e) {
 template <bool EMIT>
 __global__ void __launch_bounds__(kHThreads, 3) k_plain_block(const __grid_constant__ Job j) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     PlainSmem& ps = *reinterpret_cast<PlainSmem*>(smem_raw);
     const int64_t e = j.ev_begin + blockIdx.x;
     if (e >= j.ev_begin + j.ev_count) return;
@@ -2442,6 +2468,8 @@ __global__ void __launch_bounds__(kHThreads, 3) k_plain_block(const __grid_const
 // -------------------------------------------------------- accept bits
 
 __global__ void k_accept(const __grid_constant__ Job j) {
+    chain_next();
+    chain_wait();
     if (!j.accept_bits) return;
     const int64_t nwords = (j.n_events + 31) / 32;
     const int lane = threadIdx.x & 31;
@@ -2493,6 +2521,8 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* sh, int64
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const __grid_constant__ Job j) {
     __shared__ int64_t sh[33];
+    chain_next();
+    chain_wait();
     const int64_t n = j.n_events * j.S;
     const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -2509,6 +2539,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const __grid_const
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_top(const __grid_constant__ Job j) {
     __shared__ int64_t sh[33];
+    chain_next();
+    chain_wait();
     const int64_t n = j.n_events * j.S;
     const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
     int64_t carry = 0;
@@ -2528,6 +2560,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_top(const __grid_constant
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(const __grid_constant__ Job j) {
     __shared__ int64_t sh[33];
+    chain_next();
+    chain_wait();
     const int64_t n = j.n_events * j.S;
     const int64_t ntiles = (n + kScanTile - 1) / kScanTile;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -2556,7 +2590,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const __grid_constan
 // written by a path that did not keep the event (it moved on to the next
 // path part-way) are dropped; the final path recorded the event again.
 __global__ void k_scatter(const __grid_constant__ Job j) {
+    chain_next();
+    chain_wait();
+    // enqueued behind the count: only a record and a buffer that hold every triplet
     const unsigned long long n = j.ctrl->scratch_n;
+    if (!j.triplets || n > (unsigned long long)j.tscr_cap || j.ctrl->trip_total > j.trip_cap ||
+        (*(volatile int32_t*)&j.ctrl->status & (kStInvalid | kStNoScratch | kStNoPool)))
+        return;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += stride) {
         const TripEntry te = j.tscr[q];
@@ -2679,7 +2719,45 @@ int generic_max_blocks_per_sm(int threads) {
     return nb;
 }
 
+// Blocks of a captured kernel that can have work for this job, at most `full`:
+// small batches do not pay for the setup of grids that fill the chip (an empty
+// k_medium with its 2128 blocks takes 8 us, a one-tile scan over 304 blocks 6).
+unsigned useful_blocks(const void* f, const Job& j, unsigned full) {
+    const int64_t ne = std::max<int64_t>(j.ev_count, 1), words = (j.n_events + 31) / 32;
+    int64_t n = full;
+    if (f == (const void*)k_light<false> || f == (const void*)k_light<true>)
+        n = (ne + j.grab - 1) / j.grab;  // (a block's further warps find no event)
+    else if (f == (const void*)k_medium<false> || f == (const void*)k_heavy || f == (const void*)k_generic<false>)
+        n = ne;
+    else if (f == (const void*)k_heavy_units<false>)
+        n = ne * std::max(j.S - 1, 1);
+    else if (f == (const void*)k_heavy_final)
+        n = (ne + 7) / 8;
+    else if (f == (const void*)k_accept)
+        n = (words + 7) / 8;
+    else if (f == (const void*)k_scan_reduce || f == (const void*)k_scan_down)
+        n = (j.n_events * j.S + kScanTile - 1) / kScanTile;
+    return (unsigned)std::min<int64_t>(full, std::max<int64_t>(n, 1));
+}
+
 const void* light_count_kernel_ptr() { return (const void*)k_light<false>; }
+
+// Launches a kernel of a run behind the one before it on the stream (see
+// chain_wait): its blocks are set up while the one before drains.
+template <class A>
+static void chain_launch(void (*k)(A), unsigned grid, unsigned block, size_t smem, cudaStream_t st, const A& a) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, k, a);  // errors: cudaGetLastError of the launchers
+}
 
 // Kernels take the job by value (a __grid_constant__ parameter), so every
 // field read is a constant-bank operand rather than a load.
@@ -2697,20 +2775,20 @@ cudaError_t launch_light_count(const Job& job, int64_t n_events, const LaunchCfg
 }
 
 cudaError_t launch_count_lists(const Job& j, const LaunchCfg& lc, cudaStream_t st) {
-    k_medium<false><<<lc.medium_blocks, MedBCfg::THREADS, medium_smem_bytes(), st>>>(j);
-    k_sort_heavy<<<1, 1024, 0, st>>>(j);
-    k_heavy<<<lc.heavy_blocks, kHThreads, heavy_smem_bytes(), st>>>(j);
-    k_heavy_units<false><<<lc.heavy_blocks, kHThreads, heavy_smem_bytes(), st>>>(j);
-    k_heavy_final<<<lc.scan_blocks, 256, 0, st>>>(j);
-    k_generic<false><<<lc.generic_blocks, kGenThreads, 0, st>>>(j);
+    chain_launch(k_medium<false>, lc.medium_blocks, MedBCfg::THREADS, medium_smem_bytes(), st, j);
+    chain_launch(k_sort_heavy, 1, 1024, 0, st, j);
+    chain_launch(k_heavy, lc.heavy_blocks, kHThreads, heavy_smem_bytes(), st, j);
+    chain_launch(k_heavy_units<false>, lc.heavy_blocks, kHThreads, heavy_smem_bytes(), st, j);
+    chain_launch(k_heavy_final, lc.scan_blocks, 256, 0, st, j);
+    chain_launch(k_generic<false>, lc.generic_blocks, kGenThreads, 0, st, j);
     return cudaGetLastError();
 }
 
 cudaError_t launch_count_tail(const Job& j, const LaunchCfg& lc, cudaStream_t st) {
-    k_accept<<<lc.scan_blocks, 256, 0, st>>>(j);
-    k_scan_reduce<<<lc.scan_blocks, kScanThreads, 0, st>>>(j);
-    k_scan_top<<<1, kScanThreads, 0, st>>>(j);
-    k_scan_down<<<lc.scan_blocks, kScanThreads, 0, st>>>(j);
+    chain_launch(k_accept, lc.scan_blocks, 256, 0, st, j);
+    chain_launch(k_scan_reduce, lc.scan_blocks, kScanThreads, 0, st, j);
+    chain_launch(k_scan_top, 1, kScanThreads, 0, st, j);
+    chain_launch(k_scan_down, lc.scan_blocks, kScanThreads, 0, st, j);
     return cudaGetLastError();
 }
 
@@ -2769,7 +2847,7 @@ cudaError_t launch_plain_emit(const Job& j, const LaunchCfg& lc, cudaStream_t st
 }
 
 cudaError_t launch_scatter(const Job& j, const LaunchCfg& lc, cudaStream_t st) {
-    k_scatter<<<lc.scan_blocks, 256, 0, st>>>(j);
+    chain_launch(k_scatter, lc.scan_blocks, 256, 0, st, j);
     return cudaGetLastError();
 }
 
@@ -2947,9 +3025,9 @@ cudaError_t launch_window_ranges(const WinJob& w, cudaStream_t st) {
     j.block_sums = w.block_sums;
     j.trip_off = w.woff;
     j.ctrl = w.ctrl;
-    k_scan_reduce<<<w.n_sm * 2, kScanThreads, 0, st>>>(j);
-    k_scan_top<<<1, kScanThreads, 0, st>>>(j);
-    k_scan_down<<<w.n_sm * 2, kScanThreads, 0, st>>>(j);
+    chain_launch(k_scan_reduce, w.n_sm * 2, kScanThreads, 0, st, j);
+    chain_launch(k_scan_top, 1, kScanThreads, 0, st, j);
+    chain_launch(k_scan_down, w.n_sm * 2, kScanThreads, 0, st, j);
     return cudaGetLastError();
 }
 
@@ -3050,7 +3128,6 @@ extern "C" jpsi_status jpsi_select_noalloc(const jpsi_params* p, const jpsi_batc
         if ((double)f < kk) f = std::nextafter(f, INFINITY);
         j.K = f;
     }
-    j.grab = 2;
     j.cap_small = SmallCfg::LAYER_CAP;
     j.cap_medium = MediumCfg::LAYER_CAP;
     j.persistent = 1;
@@ -3068,6 +3145,7 @@ extern "C" jpsi_status jpsi_select_noalloc(const jpsi_params* p, const jpsi_batc
     const int wpb = 4;
     const int per_sm = light_max_blocks_per_sm(wpb);
     if (per_sm < 1) return JPSI_ECUDA;
+    j.grab = b->n_events > (int64_t)4 * wpb * n_sm * per_sm ? 2 : 1;  // (as for contexts)
     if (cudaMemsetAsync(dctrl, 0, sizeof(Ctrl), st) != cudaSuccess) return JPSI_ECUDA;  // counters start at zero
     k_light<false><<<n_sm * per_sm, 32 * wpb, light_smem_bytes(wpb), st>>>(j);
     if (cudaGetLastError() != cudaSuccess) return JPSI_ECUDA;
