@@ -12,8 +12,9 @@
 //              and searches the other stations for compatible triplets (P2).
 //              Limits: 192 hits per layer, 384 per station, 32 passing trigger
 //              triplets.
-//   k_medium   the block-tile code on 2-warp blocks (384 hits per layer, 960
-//              per station, 16 x 32 cells) for the events k_light passes on.
+//   k_medium   the same sieve, with larger maps and one more pass, on 4-warp
+//              blocks (384 hits per layer, 960 per station) for the events
+//              k_light passes on.
 //   k_heavy, k_heavy_units, k_heavy_final
 //              8-warp blocks on the block tile (2048 hits per layer, 5632 per
 //              station, 32 x 64 cells), the warps taking L0 rounds and
@@ -73,13 +74,13 @@ struct SmallCfg {
     static constexpr int TCAP = 32;                 // passing trigger triplets kept (CHAIN)
     static constexpr uint8_t CLS = kClsLight;       // event class of this path
 };
-// the size limits of the medium tile (a 2-warp block tile, MedBCfg below)
+// the size limits of the medium path (MediumTile below)
 struct MediumCfg {
     static constexpr int LAYER_CAP = 384, HCAP = 960;
     static constexpr uint8_t CLS = kClsMedium;
 };
 
-// block-tile paths: a block of THREADS threads stages a station (each thread
+// block-tile path: a block of THREADS threads stages a station (each thread
 // up to RMAX hits per layer) into NY x NX cells per layer, and its warps
 // share the station's enumeration rounds and trigger-slope searches
 template <int THREADS_, int RMAX_, int HCAP_, int NX_, int NY_, uint8_t CLS_>
@@ -93,8 +94,6 @@ struct BCfg {
 };
 // the block tile proper: 8 warps, 2048 hits per layer, 5632 per station, 32 x 64 cells
 using HeavyCfg = BCfg<256, 8, 5632, 64, 32, kClsHeavy>;
-// the medium tile: 2 warps, 384 hits per layer, 960 per station, 16 x 32 cells
-using MedBCfg = BCfg<64, 6, 960, 32, 16, kClsMedium>;
 constexpr int kHThreads = HeavyCfg::THREADS;
 constexpr int kHLayerCap = HeavyCfg::LAYER_CAP;
 constexpr int kHHCap = HeavyCfg::HCAP;
@@ -125,9 +124,11 @@ struct TileView {
 constexpr int kMapRows = 128;             // a map has 128 rows (s_y) of 64 columns (s_x), both modulo
 constexpr int kMapWords = 2 * kMapRows;   // word 2 y + (x >> 5), bit x
 struct WarpTile {
+    static constexpr int TCAP = SmallCfg::TCAP;
+    static constexpr uint8_t CLS = kClsLight;
     float2 P[SmallCfg::HCAP + 32];        // (s_x, s_y); reads run up to 31 places past the last hit
     alignas(16) uint32_t map[2][kMapWords];
-    uint32_t pend[64];                    // triples: station << 24 | i << 16 | j << 8 | k
+    uint32_t pend[64];                    // triples: station << 27 | i << 18 | j << 9 | k
     uint8_t left[2][SmallCfg::LAYER_CAP]; // layer-local indices of the hits that the sieve leaves
     int32_t off[3 * kMaxStations + 1];    // the event's offsets
     int32_t count[kMaxStations];          // passing triplets per station
@@ -138,6 +139,30 @@ struct WarpTile {
     };
     uint8_t alive[SmallCfg::TCAP];
     static_assert(SmallCfg::LAYER_CAP <= 256, "8-bit indices");
+};
+
+// The same for the four warps of a medium block (384 hits per layer, 960 per
+// station): maps of 128 columns, what is left of all three layers, and pending
+// triples for each warp.
+struct MediumTile {
+    static constexpr int THREADS = 128, WARPS = THREADS / 32, BLOCKS = 8, TCAP = kTCap;
+    static constexpr uint8_t CLS = kClsMedium;
+    float2 P[MediumCfg::HCAP + THREADS];
+    alignas(16) uint32_t map[2][4 * kMapRows];  // word 4 y + (x >> 5), bit x
+    uint32_t pend[WARPS][64];
+    uint16_t left[3][MediumCfg::LAYER_CAP];
+    int n_left[3];
+    int32_t off[3 * kMaxStations + 1];
+    int32_t count[kMaxStations];
+    int red[WARPS][3];                          // largest |slope|, largest and smallest 1/z (bit patterns)
+    int s_gi, s_flag;
+    float2 T[TCAP];
+    union {
+        unsigned long long Tijk[TCAP];
+        float2 Tt[TCAP];
+    };
+    uint8_t alive[TCAP];
+    static_assert(MediumCfg::LAYER_CAP <= 512, "9-bit indices in pend");
 };
 
 template <class B>
@@ -376,17 +401,11 @@ __device__ int stage_layer_block(const Job& j, BlockSmem<B>& sm, int l, int32_t 
     if (lane == 31) sm.wsum[wp] = incl;
     __syncthreads();
     int woff = 0, total = 0;
-    if constexpr (B::WARPS > 2) {  // the warps' offsets by a scan over the lanes
+    {  // the warps' offsets by a scan over the lanes
         const int ws = lane < B::WARPS ? sm.wsum[lane] : 0;
         const int wi = warp_incl_scan(ws, lane);
         woff = __shfl_sync(kFull, wi - ws, wp);
         total = __shfl_sync(kFull, wi, B::WARPS - 1);
-    } else {
-#pragma unroll
-        for (int q = 0; q < B::WARPS; ++q) {
-            woff += q < wp ? sm.wsum[q] : 0;
-            total += sm.wsum[q];
-        }
     }
     int run = pbase + woff + incl - cnt;
 #pragma unroll
@@ -1022,14 +1041,14 @@ __device__ __forceinline__ void sieve_dilate(uint32_t* map, const uint32_t* othe
     __syncwarp();
 }
 
-// P1 on the event's pending triples, 32 at a time, until at most `keep` of its np
+// P1 on the warp's pending triples, 32 at a time, until at most `keep` of its np
 // are left (their number is returned), and what follows from a pass: the
 // triplet's rank in its unit (from the station's count), its row (emit pass),
 // its slopes if it is a trigger triplet and the event keeps them (`sink`), and
 // its entry in the scatter record.
-template <bool EMIT>
-__device__ __forceinline__ int light_fit(const Job& j, WarpTile& w, int lane, const Cuts& c, int64_t e, bool sink,
-                                         int np, int keep) {
+template <bool EMIT, class W>
+__device__ __forceinline__ int light_fit(const Job& j, W& w, const uint32_t* pend, int lane, const Cuts& c, int64_t e,
+                                         bool sink, int np, int keep) {
     __syncwarp();
 #pragma unroll 1
     while (np > keep) {
@@ -1040,11 +1059,11 @@ __device__ __forceinline__ int light_fit(const Job& j, WarpTile& w, int lane, co
         float2 tt = make_float2(0.f, 0.f);
         int st = 0, ii = 0, jj = 0, kk = 0;
         if (lane < n) {
-            const uint32_t en = w.pend[first + lane];
-            st = en >> 24;
-            ii = (en >> 16) & 0xff;
-            jj = (en >> 8) & 0xff;
-            kk = en & 0xff;
+            const uint32_t en = pend[first + lane];
+            st = en >> 27;
+            ii = (en >> 18) & 511;
+            jj = (en >> 9) & 511;
+            kk = en & 511;
             const int32_t h0 = w.off[3 * st] + ii, h1 = w.off[3 * st + 1] + jj, h2 = w.off[3 * st + 2] + kk;
             const float xs[3] = {__ldg(j.x + h0), __ldg(j.x + h1), __ldg(j.x + h2)};
             const float ys[3] = {__ldg(j.y + h0), __ldg(j.y + h1), __ldg(j.y + h2)};
@@ -1058,7 +1077,7 @@ __device__ __forceinline__ int light_fit(const Job& j, WarpTile& w, int lane, co
         int rank = 0;
         if (ok) {
             rank = atomicAdd(&w.count[st], 1);
-            if (sink && st == j.trig && rank < SmallCfg::TCAP) {
+            if (sink && st == j.trig && rank < W::TCAP) {
                 w.T[rank] = make_float2(mx, my);
                 if (j.distinct) w.Tijk[rank] = pack_ijk(ii, jj, kk);
                 if (kStream) w.Tt[rank] = tt;
@@ -1086,7 +1105,7 @@ __device__ __forceinline__ int light_fit(const Job& j, WarpTile& w, int lane, co
                     te.unit = (int32_t)(e * j.S + st);
                     te.rank = rank;
                     te.ijk = (unsigned long long)ii | ((unsigned long long)jj << 20) | ((unsigned long long)kk << 40) |
-                             ((unsigned long long)kClsLight << kTagShift);
+                             ((unsigned long long)W::CLS << kTagShift);
                     j.tscr[b] = te;
                 }
             }
@@ -1210,22 +1229,24 @@ __device__ __forceinline__ void sieve_layers(const Job& j, WarpTile& w, int lane
 }
 
 // The triples whose pairs are all close enough, among the hits that the sieve
-// left of layers 0 and 2 and all of layer 1 (128 hits at a time in registers): each
-// hit of layer 2 against layer 1, each pair found against layer 0.  They join the
-// event's pending triples (np), which are fitted 32 at a time, or at the end of
-// the station when `all` is set: the fits of an event's non-trigger stations
-// share their instructions.
-template <bool EMIT>
-__device__ __forceinline__ void sieve_triples(const Job& j, WarpTile& w, int lane, const Cuts& c, float B, int64_t e,
-                                              int s, int s1, int n1, int s2, int m0, int m2, bool sink, bool all,
-                                              int& np) {
+// left of layers 0 (l0[0, m0)) and 2 (l2[0, m2)) and of layer 1 (l1[0, m1), or all
+// its m1 hits when l1 is null), 128 of them at a time in registers: each hit k_first +
+// i k_step of l2 against layer 1, each pair found against l0.  They join the warp's
+// pending triples (np), which are fitted 32 at a time, or at the end of the station
+// when `all` is set: the fits of an event's non-trigger stations share their
+// instructions.
+template <bool EMIT, bool FILTER, class W, class L>
+__device__ __forceinline__ void sieve_triples(const Job& j, W& w, uint32_t* pend, int lane, const Cuts& c, float B,
+                                              int64_t e, int s, int s1, int s2, const L* l0, int m0, const L* l1,
+                                              int m1, const L* l2, int m2, int k_first, int k_step, bool sink,
+                                              bool all, int& np) {
     const uint32_t lt = (1u << lane) - 1u;
-    const int hi0 = w.left[0][min(lane, max(m0 - 1, 0))];  // what is left of layer 0, its first 32
+    const int hi0 = l0[min(lane, max(m0 - 1, 0))];  // what is left of layer 0, its first 32
     const float2 Pi0 = w.P[m0 > 0 ? hi0 : 0];
     float2 Pj[4], Pk = make_float2(0.f, 0.f), Q = Pk;
-    int j0 = -128, k = m2, hk = 0, hj = 0, i0 = m0;  // next: layer 0 from i0 on for the pair (hj, hk)
+    int j0 = -128, k = m2 + k_step, hk = 0, hj = 0, i0 = m0;  // next: layer 0 from i0 on for the pair (hj, hk)
     unsigned mine = 0;                               // this lane's rounds with further partners of hk
-    bool more = m2 > 0;
+    bool more = m2 > k_first;
     for (;;) {
 #pragma unroll 1
         while (more && np <= 32) {
@@ -1235,26 +1256,29 @@ __device__ __forceinline__ void sieve_triples(const Job& j, WarpTile& w, int lan
                     const int from = __ffs(lanes) - 1;
                     hj = j0 + 32 * (__ffs(__shfl_sync(kFull, mine, from)) - 1) + from;
                     if (lane == from) mine &= mine - 1;
-                    if (hj < n1) {  // (an infinite bound lets the places past the end through)
+                    if (hj < m1) {  // (an infinite bound lets the places past the end through)
+                        if (FILTER && l1) hj = l1[hj];
                         Q = w.P[s1 + hj];
                         i0 = 0;
                     }
                 } else {
-                    if (++k >= m2) {  // the next 128 hits of layer 1
+                    k += k_step;
+                    if (k >= m2) {  // the next 128 hits of layer 1
                         j0 += 128;
-                        if (j0 >= n1) {
+                        if (j0 >= m1) {
                             more = false;
                             continue;
                         }
-                        k = 0;
+                        k = k_first;
 #pragma unroll
                         for (int r = 0; r < 4; ++r) {
                             const int p = j0 + 32 * r + lane;
-                            Pj[r] = w.P[s1 + min(p, n1 - 1)];
-                            if (p >= n1) Pj[r].x = INFINITY;
+                            const int h = min(p, m1 - 1);
+                            Pj[r] = w.P[s1 + (FILTER && l1 ? (int)l1[h] : h)];
+                            if (p >= m1) Pj[r].x = INFINITY;
                         }
                     }
-                    hk = w.left[1][k];
+                    hk = l2[k];
                     Pk = w.P[s2 + hk];
 #pragma unroll
                     for (int r = 0; r < 4; ++r) mine |= pair_ok(Pj[r].x, Pj[r].y, Pk.x, Pk.y, B) ? 1u << r : 0u;
@@ -1264,7 +1288,7 @@ __device__ __forceinline__ void sieve_triples(const Job& j, WarpTile& w, int lan
             int hi = hi0;
             float2 Pi = Pi0;
             if (i0 > 0) {
-                hi = w.left[0][min(i0 + lane, m0 - 1)];
+                hi = l0[min(i0 + lane, m0 - 1)];
                 Pi = w.P[hi];
             }
             const bool cand =
@@ -1272,12 +1296,12 @@ __device__ __forceinline__ void sieve_triples(const Job& j, WarpTile& w, int lan
             const unsigned mask = __ballot_sync(kFull, cand);
             const int at = np + __popc(mask & lt);
             if (cand && JPSI_IN(j.ctrl, at < 64))
-                w.pend[at] = (uint32_t)s << 24 | (uint32_t)hi << 16 | (uint32_t)hj << 8 | (uint32_t)hk;
+                pend[at] = (uint32_t)s << 27 | (uint32_t)hi << 18 | (uint32_t)hj << 9 | (uint32_t)hk;
             np += __popc(mask);
             i0 += 32;
         }
         np = uniform(np);
-        np = light_fit<EMIT>(j, w, lane, c, e, sink, np, all && !more ? 0 : 32);
+        np = light_fit<EMIT>(j, w, pend, lane, c, e, sink, np, all && !more ? 0 : 32);
         if (!more) break;
     }
 }
@@ -1313,7 +1337,9 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
     static_assert(SmallCfg::LAYER_CAP <= 6 * 32, "rounds of a layer");
     m2 = uniform(m2);
     m0 = uniform(m0);
-    if (m2 > 0 || (all && np > 0)) sieve_triples<EMIT>(j, w, lane, c, sb.B, e, s, n0, n1, n0 + n1, m0, m2, sink, all, np);
+    if (m2 > 0 || (all && np > 0))
+        sieve_triples<EMIT, false>(j, w, w.pend, lane, c, sb.B, e, s, n0, n0 + n1, w.left[0], m0,
+                                   (const uint8_t*)nullptr, n1, w.left[1], m2, 0, 1, sink, all, np);
     return 0;
 }
 
@@ -1321,7 +1347,8 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
 // slopes (mx, my)?  The warp tests the tube on 32 hits a step; every hit of
 // layer 0 that passes it is tried with every such hit of layer 1, and those
 // pairs with 32 hits of layer 2 a step (P1 and P2).  Warp-uniform.
-__device__ bool sieve_road(const Job& j, const WarpTile& w, int lane, const Cuts& c, const StationBounds& sb,
+template <class W>
+__device__ bool sieve_road(const Job& j, const W& w, int lane, const Cuts& c, const StationBounds& sb,
                            int32_t o0, int n0, int n1, int n2, float mx, float my, float2 Tt) {
     const int s1 = n0, s2 = n0 + n1, n = s2 + n2;
     // the hits of places [p0, p0 + 32) of a layer ending at `end` that pass the tube
@@ -1619,7 +1646,6 @@ __device__ __forceinline__ void heavy_to_generic(const Job& j, int gi, int64_t e
 // Who hands an event on when a station cannot be pruned: gi >= 0 is the
 // event's block-tile list entry (its state in Job::hT);
 constexpr int kGiPlain = -1;  // the one-launch form: the same block goes on unpruned
-constexpr int kGiOwn = -2;    // a block that owns the whole event: to the unpruned list
 
 // Pulls the hit lines of station s of the event in sm.off into L2 (block
 // version of prefetch_hits_l2; addresses stay inside [o[0] & ~31, o[3])).
@@ -1657,8 +1683,6 @@ __device__ bool heavy_unit(const Job& j, BlockSmem<B>& sm, const Cuts& c, int gi
                 j.ev_class[e] = kClsInvalid;
             } else if (gi == kGiPlain) {
                 j.ev_class[e] = kClsGeneric;
-            } else if (gi == kGiOwn) {
-                push_event(j, e, kClsGeneric);
             } else {
                 heavy_to_generic(j, gi, e);
             }
@@ -1787,107 +1811,281 @@ __device__ void heavy_event(const Job& j, HeavySmem& sm, const Cuts& c, int gi, 
     }
 }
 
-// Medium tile: 2-warp blocks take the events of the medium list, one at a
-// time, and run every station of their event: the trigger station first (in
-// CHAIN mode its passing triplets' slopes, at most kTCap, stay in shared
-// memory), then the others, whose enumeration rounds share the warps with
-// the searches for those slopes.  An event with more trigger slopes goes on
-// to the block tile; one with extreme coordinates to the unpruned kernel.
-struct MediumSmem {
-    BlockSmem<MedBCfg> b;
-    float2 T[kTCap];
-    union {
-        unsigned long long Tijk[kTCap];  // their packed hits (distinct_hits)
-        float2 Tt[kTCap];                // or their (min t, max t) (free-streaming windows)
-    };
-    uint8_t alive[kTCap];
-};
+// Medium path: 4-warp blocks take the events of the medium list, one at a time, and
+// run every station of their event with the sieve of the warp path, shared by the
+// warps: the trigger station first (in CHAIN mode its passing triplets'
+// slopes, at most kTCap, stay in shared memory), then the others and the searches
+// for those slopes.  An event with more trigger slopes goes on to the block tile;
+// one with extreme coordinates to the unpruned kernel.
+//   Bound by instruction issue and the barriers between the maps.  The events of
+// a 55 000-event log-normal timeslice: 379 us with cell-sorted tiles, 280 with
+// the sieve; of 100 000 free-streaming collisions: 1.23 -> 1.02 ms.  Four warps and
+// eight blocks per SM (64 registers) against two warps and 13 blocks: the same
+// on the timeslice, 4 % slower on the collisions, but an event takes little more than
+// half as long: medium and block tiles of 1 000 collisions 161 -> 131 us, of 10 000
+// log-normal events 363 -> 336 us.
 
-template <bool EMIT>
-__device__ void medium_event(const Job& j, MediumSmem& ms, const Cuts& c, int64_t e) {
-    BlockSmem<MedBCfg>& sm = ms.b;
+__device__ __forceinline__ SieveBit medium_bit(float2 s, float inv) {
+    const int cx = sieve_cell(s.x, inv), cy = sieve_cell(s.y, inv);
+    return {((cy & (kMapRows - 1)) << 2) + ((cx >> 5) & 3), __funnelshift_l(0u, 1u, cx)};
+}
+
+// sieve_dilate for the block: a ring of 128 columns; each thread has RT consecutive
+// rows.  With MEET, `other` is cleared behind it.
+template <bool MEET>
+__device__ __forceinline__ void medium_dilate(uint32_t* map, uint32_t* other) {
+    constexpr int RT = kMapRows / MediumTile::THREADS;
+    const int t = RT * threadIdx.x;
+    __syncthreads();
+    uint4* m4 = reinterpret_cast<uint4*>(map);
+    uint4 q[RT + 2];
+#pragma unroll
+    for (int r = 0; r < RT + 2; ++r) q[r] = m4[(t + r + kMapRows - 1) & (kMapRows - 1)];
+    uint32_t d[RT][4];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+        const uint4 a = q[r], b = q[r + 1], c = q[r + 2];
+        const uint32_t v[4] = {a.x | b.x | c.x, a.y | b.y | c.y, a.z | b.z | c.z, a.w | b.w | c.w};
+        uint4 o = make_uint4(~0u, ~0u, ~0u, ~0u);
+        if (MEET) {
+            uint4* o4 = reinterpret_cast<uint4*>(other);
+            o = o4[t + r];
+            o4[t + r] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        const uint32_t ov[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            d[r][i] = (v[i] | __funnelshift_l(v[(i + 3) & 3], v[i], 1) | __funnelshift_r(v[i], v[(i + 1) & 3], 1)) & ov[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RT; ++r) m4[t + r] = make_uint4(d[r][0], d[r][1], d[r][2], d[r][3]);
+    __syncthreads();
+}
+
+// The hits of a layer (places [p0, p0 + n)) whose cells are set in `map`: their
+// layer-local indices to `left` (any order), their cells to `mark` (if given).
+__device__ __forceinline__ void medium_pass(const Job& j, MediumTile& w, float inv, int p0, int n, const uint32_t* map,
+                                            uint32_t* mark, uint16_t* left, int* n_left) {
+    constexpr int T = MediumTile::THREADS, R = MediumCfg::LAYER_CAP / T;
     const int tid = threadIdx.x, lane = tid & 31;
-    const int S = j.S;
-    const bool chain = j.mode == 1 && S > 1;
-    const int nproc = j.mode == 1 ? S : 1;
-    load_event_offsets(j, sm, e);
-    if (EMIT) {
-        for (int si = 0; si < nproc; ++si) {
-            const int s = station_of(si, j.trig);
-            if (j.unit_counts[e * S + s] == 0) continue;
-            TSink ts{false, nullptr, 0, nullptr, 0};
-            int cnt = 0;
-            heavy_unit<true>(j, sm, c, kGiOwn, e, s, ts, nullptr, nullptr, 0, cnt,
-                             si + 1 < nproc ? station_of(si + 1, j.trig) : -1);
-            __syncthreads();
-        }
-        return;
+    const uint32_t lt = (1u << lane) - 1u;
+    unsigned bits = 0;
+    int m = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (T * r >= n) break;  // block-uniform
+        const SieveBit b = medium_bit(w.P[p0 + T * r + tid], inv);
+        const bool in = (T * r + tid < n) & ((map[b.word] & b.bit) != 0);
+        if (mark && in) atomicOr(&mark[b.word], b.bit);
+        bits |= in ? 1u << r : 0u;
+        m += __popc(__ballot_sync(kFull, in));
     }
-    int trig_count = 0, nT = 0;
-    for (int si = 0; si < nproc; ++si) {
-        const int s = station_of(si, j.trig);
-        if (tid == 0) sm.s_nT = 0;
-        __syncthreads();
-        TSink ts{(chain || j.distinct) && si == 0, ms.T, kTCap, &sm.s_nT, 0};
-        ts.ijk = j.distinct ? ms.Tijk : nullptr;
-        ts.tt = kStream ? ms.Tt : nullptr;
-        int cnt = 0;
-        const int sn = si + 1 < nproc ? station_of(si + 1, j.trig) : -1;
-        if (!heavy_unit<false>(j, sm, c, kGiOwn, e, s, ts, ms.T, ms.alive, si == 0 ? 0 : nT, cnt, sn,
-                               kStream ? ms.Tt : nullptr))
-            return;
-        __syncthreads();
-        if (si > 0) continue;
-        trig_count = cnt;
-        nT = sm.s_nT;
-        if (nT > kTCap) {  // more trigger slopes than this tile keeps
-            if (tid == 0) push_event(j, e, kClsHeavy);
-            return;
-        }
-        if (!chain) break;
-        for (int i = tid; i < nT; i += MedBCfg::THREADS) ms.alive[i] = 1;
-        __syncthreads();
-    }
-    int tc = trig_count;
-    if (chain) {
-        if (tid == 0) sm.s_cand = 0;
-        __syncthreads();
-        int a = 0;
-        for (int ti = tid; ti < nT; ti += MedBCfg::THREADS) a += ms.alive[ti];
-        a = __reduce_add_sync(kFull, a);
-        if (lane == 0 && a) atomicAdd(&sm.s_cand, a);
-        __syncthreads();
-        tc = sm.s_cand;
-    }
-    if (j.distinct) {
-        const bool f = nT >= 2 && block_disjoint_pair<MedBCfg::THREADS>(ms.Tijk, chain ? ms.alive : nullptr, nT,
-                                                                         &sm.s_hx);
-        if (tid == 0) j.dpair[e] = f;
-    }
-    if (tid == 0) {
-        if (j.mode == 0)
-            for (int s = 0; s < S; ++s)
-                if (s != j.trig) j.unit_counts[e * S + s] = 0;
-        j.track_counts[e] = tc;
+    int at = 0;
+    if (lane == 0 && m) at = atomicAdd(n_left, m);
+    at = __shfl_sync(kFull, at, 0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (T * r >= n) break;
+        const unsigned mask = __ballot_sync(kFull, bits >> r & 1u);
+        const int i = at + __popc(mask & lt);
+        if ((bits >> r & 1u) && JPSI_IN(j.ctrl, i < MediumCfg::LAYER_CAP)) left[i] = (uint16_t)(T * r + tid);
+        at += __popc(mask);
     }
 }
 
+// Stages station s of the event in w.off and finds its triples (see
+// sieve_layers; a third map leaves fewer hits of layer 1 when layer 2 has more
+// than kFilterMin).  Returns 0, 1 for a hit with z <= 0 or 2 for one whose
+// pruning bound is not finite; block-uniform, all threads call it.
+constexpr int kFilterMin = 8;
 template <bool EMIT>
-__global__ void __launch_bounds__(MedBCfg::THREADS, 14) k_medium(const __grid_constant__ Job j) {
+__device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const Cuts& c, int64_t e, int s, bool sink,
+                                              bool all, StationBounds& sb, int& np) {
+    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+    const int32_t o0 = uniform(w.off[3 * s]);
+    const int n0 = uniform(w.off[3 * s + 1]) - o0, n1 = uniform(w.off[3 * s + 2]) - o0 - n0,
+              n2 = uniform(w.off[3 * s + 3]) - o0 - n0 - n1, n = n0 + n1 + n2;
+    const int s1 = n0, s2 = n0 + n1;
+    constexpr int T = MediumTile::THREADS;
+    float smax = 0.0f, rmax = 0.0f, rmin = INFINITY;
+    for (int p0 = 0; p0 < n; p0 += 4 * T) {
+        float x[4], y[4], z[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (p0 + T * q < n) {  // block-uniform; threads past the end read the last hit again
+                const int32_t h = o0 + min(p0 + T * q + tid, n - 1);
+                x[q] = __ldg(j.x + h);
+                y[q] = __ldg(j.y + h);
+                z[q] = __ldg(j.z + h);
+            }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (p0 + T * q < n) {
+                const float iz = rcp_approx(z[q]);
+                const float2 v = make_float2(__fmul_rn(x[q], iz), __fmul_rn(y[q], iz));
+                smax = max3_abs_nan(smax, v.x, v.y);
+                rmax = max3_abs_nan(rmax, iz, 0.0f);
+                rmin = fminf(rmin, iz);
+                if (p0 + T * q + tid < n) w.P[p0 + T * q + tid] = v;
+            }
+    }
+    auto reduce = [&]() {  // the block's maxima, minimum, and what they say of the hits
+        const int si = __reduce_max_sync(kFull, __float_as_int(smax)), ri = __reduce_max_sync(kFull, __float_as_int(rmax)),
+                  ni = __reduce_min_sync(kFull, __float_as_int(rmin));
+        if (lane == 0) {
+            w.red[wp][0] = si;
+            w.red[wp][1] = ri;
+            w.red[wp][2] = ni;
+        }
+        __syncthreads();
+        const int wl = lane & (MediumTile::WARPS - 1);
+        const int bs = __reduce_max_sync(kFull, w.red[wl][0]), br = __reduce_max_sync(kFull, w.red[wl][1]),
+                  bn = __reduce_min_sync(kFull, w.red[wl][2]);
+        smax = __int_as_float(bs);
+        rmax = __int_as_float(br);
+        sb = station_bounds(rmax, smax, j.K);
+        return bs < 0x7f800000 && br < 0x7e800000 && bn > 0x00800000 && sb.B < INFINITY;
+    };
+    uint32_t *ma = w.map[0], *mb = w.map[1];
+#pragma unroll
+    for (int q = 0; q < 2 * kMapRows / T; ++q) reinterpret_cast<uint4*>(w.map)[T * q + tid] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < 3) w.n_left[tid] = 0;
+    if (!uniform(reduce())) {  // some odd coordinate: classify every hit exactly (see sieve_classify)
+        bool zbad = false, wild = false;
+        smax = rmax = 0.0f;
+        for (int p = tid; p < n; p += T) {
+            const HitPrep h = hit_prep(__ldg(j.x + o0 + p), __ldg(j.y + o0 + p), __ldg(j.z + o0 + p), j.K);
+            zbad |= h.zbad;
+            wild |= h.wild;
+            const bool live = h.live & !h.wild;
+            w.P[p] = live ? make_float2(h.sx, h.sy) : make_float2(INFINITY, INFINITY);
+            if (live) {
+                smax = fmaxf(smax, fmaxf(fabsf(h.sx), fabsf(h.sy)));
+                rmax = fmaxf(rmax, h.r);
+            }
+        }
+        if (uniform(__syncthreads_or(zbad))) return 1;
+        if (uniform(__syncthreads_or(wild))) return 2;
+        reduce();
+    }
+    for (int p0 = 0; p0 < n1; p0 += T) {
+        const SieveBit b = medium_bit(w.P[s1 + p0 + tid], sb.inv);
+        if (p0 + tid < n1) atomicOr(&ma[b.word], b.bit);
+    }
+    medium_dilate<false>(ma, nullptr);
+    medium_pass(j, w, sb.inv, 0, n0, ma, mb, w.left[0], &w.n_left[0]);
+    medium_dilate<true>(mb, ma);
+    medium_pass(j, w, sb.inv, s2, n2, mb, ma, w.left[2], &w.n_left[2]);
+    __syncthreads();
+    const int m0 = uniform(w.n_left[0]), m2 = uniform(w.n_left[2]);
+    int m1 = n1;
+    const uint16_t* l1 = nullptr;
+    if (m2 > kFilterMin) {
+        medium_dilate<true>(ma, mb);
+        medium_pass(j, w, sb.inv, s1, n1, ma, nullptr, w.left[1], &w.n_left[1]);
+        __syncthreads();
+        m1 = uniform(w.n_left[1]);
+        l1 = w.left[1];
+    }
+    sieve_triples<EMIT, true>(j, w, w.pend[wp], lane, c, sb.B, e, s, s1, s2, w.left[0], m0, l1, m1, w.left[2], m2, wp,
+                              MediumTile::WARPS, sink, all, np);
+    return 0;
+}
+
+template <bool EMIT>
+__device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t e) {
+    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+    const int S = j.S;
+    const bool chain = j.mode == 1 && S > 1;
+    const int nproc = j.mode == 1 ? S : 1;
+    for (int i = tid; i <= 3 * S; i += MediumTile::THREADS) w.off[i] = __ldg(j.off + e * 3 * S + i);
+    if (tid < kMaxStations) w.count[tid] = 0;
+    __syncthreads();
+    int np = 0, nT = 0;
+    const bool sink = !EMIT && (chain || j.distinct);
+#pragma unroll 1
+    for (int si = 0; si < nproc; ++si) {
+        const int s = station_of(si, j.trig);
+        const int cnt = EMIT ? uniform(j.unit_counts[e * S + s]) : 0;
+        if (EMIT && cnt == 0) continue;
+        if (!j.host_hits && wp == 0) {  // the next station's lines start towards L2
+            if (si == 0) prefetch_hits_l2(j, w.off[3 * s], w.off[3 * s + 3], lane);
+            if (si + 1 < nproc) {
+                const int sn = station_of(si + 1, j.trig);
+                prefetch_hits_l2(j, w.off[3 * sn], w.off[3 * sn + 3], lane);
+            }
+        }
+        StationBounds sb;
+        const int st = medium_station<EMIT>(j, w, c, e, s, sink, EMIT || (sink && si == 0) || si + 1 == nproc, sb, np);
+        if (EMIT) {
+            __syncthreads();
+            if ((st != 0 || w.count[s] != cnt) && tid == 0) atomicOr(&j.ctrl->status, kStEmitMismatch);
+            continue;
+        }
+        if (st != 0) {
+            if (tid == 0) {
+                if (st == 1) {
+                    atomicOr(&j.ctrl->status, kStInvalid);
+                    j.ev_class[e] = kClsInvalid;
+                } else {
+                    push_event(j, e, kClsGeneric);
+                }
+            }
+            return;
+        }
+        if (si == 0) {
+            __syncthreads();
+            nT = sink ? uniform(w.count[s]) : 0;
+            if (nT > kTCap) {  // more trigger slopes than this path keeps
+                if (tid == 0) push_event(j, e, kClsHeavy);
+                return;
+            }
+            if (tid < nT) w.alive[tid] = 1;
+        } else {
+            const int32_t o0 = w.off[3 * s];
+            const int n0 = w.off[3 * s + 1] - o0, n1 = w.off[3 * s + 2] - o0 - n0, n2 = w.off[3 * s + 3] - o0 - n0 - n1;
+#pragma unroll 1
+            for (int ti = wp; ti < nT; ti += MediumTile::WARPS) {  // (CHAIN only: PAPER has one station)
+                if (!w.alive[ti]) continue;
+                const float2 m = w.T[ti];
+                const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, m.x, m.y,
+                                              kStream ? w.Tt[ti] : make_float2(0.f, 0.f));
+                __syncwarp();
+                if (!found && lane == 0) w.alive[ti] = 0;
+            }
+        }
+        __syncthreads();  // the tile may be staged again
+    }
+    if (EMIT) return;
+    static_assert(kTCap <= MediumTile::THREADS, "one flag per thread");
+    if (tid < S) j.unit_counts[e * S + tid] = w.count[tid];
+    int tc = w.count[j.trig];
+    if (chain) tc = __syncthreads_count(tid < nT && w.alive[tid]);
+    if (j.distinct) {
+        const bool f =
+            nT >= 2 && block_disjoint_pair<MediumTile::THREADS>(w.Tijk, chain ? w.alive : nullptr, nT, &w.s_flag);
+        if (tid == 0) j.dpair[e] = f;
+    }
+    if (tid == 0) j.track_counts[e] = tc;
+}
+
+template <bool EMIT>
+__global__ void __launch_bounds__(MediumTile::THREADS, MediumTile::BLOCKS) k_medium(const __grid_constant__ Job j) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     chain_wait();
-    MediumSmem& ms = *reinterpret_cast<MediumSmem*>(smem_raw);
+    MediumTile& w = *reinterpret_cast<MediumTile*>(smem_raw);
     const Cuts c{j.cx, j.cy, j.K};
     const int n_med = *(volatile int32_t*)&j.ctrl->n_medium, m0 = *(volatile int32_t*)&j.ctrl->m_begin;
     unsigned long long* ctr = &j.ctrl->work[EMIT ? 5 : 1];
     for (;;) {
-        if (threadIdx.x == 0) ms.b.s_gi = m0 + (int)atomicAdd(ctr, 1ull);
+        if (threadIdx.x == 0) w.s_gi = m0 + (int)atomicAdd(ctr, 1ull);
         __syncthreads();
-        const int gi = ms.b.s_gi;
+        const int gi = uniform(w.s_gi);
         __syncthreads();
         if (gi >= n_med) break;
-        const int64_t e = j.mlist[gi];
-        if (!EMIT || j.ev_class[e] == kClsMedium) medium_event<EMIT>(j, ms, c, e);
+        const int64_t e = uniform(j.mlist[gi]);
+        if (!EMIT || uniform(j.ev_class[e]) == kClsMedium) medium_event<EMIT>(j, w, c, e);
         __syncthreads();
     }
     chain_next();
@@ -2642,7 +2840,7 @@ __global__ void __launch_bounds__(256) k_expand_z(const int32_t* __restrict__ of
 // ------------------------------------------------------------ launchers
 
 size_t light_smem_bytes(int wpb) { return (size_t)wpb * sizeof(WarpTile); }
-static size_t medium_smem_bytes() { return sizeof(MediumSmem); }
+static size_t medium_smem_bytes() { return sizeof(MediumTile); }
 size_t heavy_smem_bytes() { return sizeof(HeavySmem); }
 static size_t plain_smem_bytes() { return sizeof(PlainSmem); }
 
@@ -2707,7 +2905,7 @@ int heavy_max_blocks_per_sm() {
 int medium_max_blocks_per_sm() {
     if (ensure_attrs() != cudaSuccess) return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_medium<false>, MedBCfg::THREADS, medium_smem_bytes()) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_medium<false>, MediumTile::THREADS, medium_smem_bytes()) !=
         cudaSuccess)
         return 0;
     return nb;
@@ -2775,7 +2973,7 @@ cudaError_t launch_light_count(const Job& job, int64_t n_events, const LaunchCfg
 }
 
 cudaError_t launch_count_lists(const Job& j, const LaunchCfg& lc, cudaStream_t st) {
-    chain_launch(k_medium<false>, lc.medium_blocks, MedBCfg::THREADS, medium_smem_bytes(), st, j);
+    chain_launch(k_medium<false>, lc.medium_blocks, MediumTile::THREADS, medium_smem_bytes(), st, j);
     chain_launch(k_sort_heavy, 1, 1024, 0, st, j);
     chain_launch(k_heavy, lc.heavy_blocks, kHThreads, heavy_smem_bytes(), st, j);
     chain_launch(k_heavy_units<false>, lc.heavy_blocks, kHThreads, heavy_smem_bytes(), st, j);
@@ -2861,7 +3059,7 @@ cudaError_t launch_emit_phase(const Job& job, int64_t n_events, const LaunchCfg&
     j.persistent = persistent ? 1 : 0;
     const int64_t nb = persistent ? lc.light_blocks : std::max<int64_t>((n_events + wpb - 1) / wpb, 1);
     k_light<true><<<(unsigned)nb, wpb * 32, smem, st>>>(j);
-    k_medium<true><<<lc.medium_blocks, MedBCfg::THREADS, medium_smem_bytes(), st>>>(j);
+    k_medium<true><<<lc.medium_blocks, MediumTile::THREADS, medium_smem_bytes(), st>>>(j);
     k_heavy_units<true><<<lc.heavy_blocks, kHThreads, heavy_smem_bytes(), st>>>(j);
     k_generic<true><<<lc.generic_blocks, kGenThreads, 0, st>>>(j);
     return cudaGetLastError();
