@@ -127,9 +127,11 @@ const Launchers kEventL{false, basek::launch_light_count, basek::launch_count_re
                         basek::launch_plain_emit, basek::useful_blocks};
 // Time inputs of a run over free-streaming windows (device pointers).
 struct StreamJob {
-    const float* t;   // [window-batch hits]
+    const float* t;   // [timeslice hits]
     const float* wb;  // [n_windows + 1]
     float dt;
+    const int32_t* shift;  // [n_windows * 3S] window batch index to timeslice index
+    int64_t n_src;         // hits of the timeslice
 };
 
 const Launchers kStreamL{true, streamk::launch_light_count, streamk::launch_count_rest, streamk::launch_emit_phase,
@@ -154,8 +156,8 @@ struct jpsi_ctx {
     RunState rs;
     // device copies for jpsi_run_host
     DevBuf hx, hy, hz, hoff, hacc, htc, htoff, htrip;
-    // window batch of a free-streaming run: ranges, their scan, offsets, hits
-    DevBuf wlo, wcnt, woff, wbs, woff32, wx, wy, wz, wt;
+    // window batch of a free-streaming run: ranges, their scan, offsets, places; z from a table
+    DevBuf wlo, wcnt, woff, wbs, woff32, wshift, wz;
     std::string last_error;
     std::mutex err_mu, cap_mu, alloc_mu;
     std::atomic<bool> timing{false};
@@ -327,7 +329,7 @@ jpsi_status prepare(jpsi_ctx* c, RunState& rs, const jpsi_batch* b, jpsi_outputs
     j.z = b->z;
     j.off = b->offsets;
     j.n_events = ne;
-    j.n_hits = b->n_hits;
+    j.n_hits = j.n_src = b->n_hits;
     j.ev_begin = 0;
     j.ev_count = ne;
     j.S = c->p.n_stations;
@@ -546,6 +548,8 @@ jpsi_status run_device(jpsi_ctx* c, RunState& rs, const jpsi_batch* b, jpsi_outp
         rs.job.dt = sj->dt;
         rs.job.t = sj->t;
         rs.job.wb = sj->wb;
+        rs.job.shift = sj->shift;
+        rs.job.n_src = sj->n_src;
     }
     const int64_t ne = b->n_events;
     cudaError_t e;
@@ -923,7 +927,9 @@ jpsi_status run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, c
         (s = ensure(c, c->wcnt, (size_t)std::max<int64_t>(n, 1) * 4, "window ranges")) ||
         (s = ensure(c, c->woff, (size_t)(n + 1) * 8, "window ranges")) ||
         (s = ensure(c, c->wbs, (size_t)((n + 4095) / 4096 + 1) * 8, "scan")) ||
-        (s = ensure(c, c->woff32, (size_t)(n + 1) * 4, "window offsets")))
+        (s = ensure(c, c->woff32, (size_t)(n + 1) * 4, "window offsets")) ||
+        (s = ensure(c, c->wshift, (size_t)std::max<int64_t>(n, 1) * 4, "window places")) ||
+        (!ts->z && (s = ensure(c, c->wz, (size_t)std::max<int64_t>(ts->n_hits, 1) * 4, "hits z"))))
         return s;
     RunState& rs = c->rs;
     WinJob w{};
@@ -945,6 +951,7 @@ jpsi_status run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, c
     w.woff = (int64_t*)c->woff.p;
     w.block_sums = (int64_t*)c->wbs.p;
     w.off_out = (int32_t*)c->woff32.p;
+    w.shift = (int32_t*)c->wshift.p;
     w.ctrl = rs.d_ctrl;
     w.n_sm = c->n_sm;
     const bool timing = c->timing.load();
@@ -959,27 +966,24 @@ jpsi_status run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, c
     const int64_t total = rs.h_ctrl->trip_total;
     if (total >= ((int64_t)1 << 31))
         return fail(c, JPSI_EINVAL, "the windows' hit ranges hold 2^31 hits or more: split the timeslice");
-    const size_t hb = (size_t)std::max<int64_t>(total, 1) * 4;
-    if ((s = ensure(c, c->wx, hb, "window hits")) || (s = ensure(c, c->wy, hb, "window hits")) ||
-        (s = ensure(c, c->wz, hb, "window hits")) || (s = ensure(c, c->wt, hb, "window hits")))
-        return s;
-    w.xo = (float*)c->wx.p;
-    w.yo = (float*)c->wy.p;
-    w.zo = (float*)c->wz.p;
-    w.to = (float*)c->wt.p;
-    if ((e = streamk::launch_window_gather(w, st)) != cudaSuccess) return cuda_fail(c, e, "window gather");
+    const bool fill_z = !ts->z && ts->n_hits > 0;
+    if ((e = streamk::launch_window_place(w, st)) != cudaSuccess) return cuda_fail(c, e, "window places");
+    if (fill_z && (e = streamk::launch_window_z(w, (float*)c->wz.p, st)) != cudaSuccess)
+        return cuda_fail(c, e, "z from geometry");
     if (timing) cudaEventRecord(rs.ev[6], st);
+    // windows in place of events: their offsets count the hits, the hits stay
+    // where they are
     jpsi_batch wbat{};
     wbat.n_events = K;
     wbat.n_hits = total;
-    wbat.x = w.xo;
-    wbat.y = w.yo;
-    wbat.z = w.zo;
+    wbat.x = ts->x;
+    wbat.y = ts->y;
+    wbat.z = ts->z ? ts->z : (const float*)c->wz.p;
     wbat.offsets = w.off_out;
-    const StreamJob sj{w.to, ts->bounds, ts->dt};
+    const StreamJob sj{ts->t, ts->bounds, ts->dt, w.shift, ts->n_hits};
     s = run_device(c, rs, &wbat, o, st, batched, false, kStreamL, &sj);
     if (s != JPSI_OK) return s;
-    int launches = kLaunchesWindows;
+    int launches = kLaunchesWindows + (fill_z ? 1 : 0);
     const bool rows = o->triplets && o->trip_needed > 0;
     if (rows) {
         if (timing) cudaEventRecord(rs.ev[7], st);
@@ -1067,7 +1071,7 @@ void jpsi_destroy(jpsi_ctx* c) {
     cudaDeviceSynchronize();
     state_free(c, c->rs);
     DevBuf* bufs[] = {&c->hx,  &c->hy,   &c->hz,  &c->hoff, &c->hacc, &c->htc, &c->htoff, &c->htrip, &c->wlo,
-                      &c->wcnt, &c->woff, &c->wbs, &c->woff32, &c->wx, &c->wy, &c->wz,   &c->wt};
+                      &c->wcnt, &c->woff, &c->wbs, &c->woff32, &c->wshift, &c->wz};
     for (DevBuf* b : bufs) release(c, *b);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);

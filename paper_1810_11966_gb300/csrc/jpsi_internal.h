@@ -86,7 +86,8 @@ struct Job {
     const float* z;
     const int32_t* off;
     int64_t n_events;             // events of the whole batch
-    int64_t n_hits;
+    int64_t n_hits;               // hits of the batch (its last offset)
+    int64_t n_src;                // hits in the arrays
     int64_t ev_begin, ev_count;   // events the warp kernels take from the batch (all by default)
     int32_t S, trig, mode, minc;
     int32_t distinct;             // distinct_hits: accept bits from dpair when minc == 2
@@ -96,7 +97,8 @@ struct Job {
     // must be coincident with the trigger triplet
     int32_t stream;
     float dt;
-    const float* t;               // [n_hits] hit times (stream)
+    const float* t;               // [n_src] hit times (stream)
+    const int32_t* shift;         // [n_events * 3S] window batch index to timeslice index (stream)
     const float* wb;              // [n_events + 1] window bounds (stream)
     float cx, cy, K;
     int32_t grab;                 // events per atomic grab (persistent light kernel)
@@ -205,7 +207,7 @@ struct WinJob {
     int64_t* woff;         // [K*3S + 1] exclusive scan of wcnt
     int64_t* block_sums;   // scan scratch
     int32_t* off_out;      // [K*3S + 1] the window batch's offsets
-    float *xo, *yo, *zo, *to;  // [total] the window batch's hits
+    int32_t* shift;        // [K*3S] from them to the timeslice's hits
     Ctrl* ctrl;            // status (kStInvalid) and trip_total = the window batch's hits
     int n_sm;
 };
@@ -213,11 +215,13 @@ namespace streamk {
 //   launch_window_ranges: validates the timeslice (times sorted per group, no
 //     NaN; z > 0 where read; bounds finite and increasing), finds each
 //     window's ranges and scans their sizes (4 launches).
-//   launch_window_gather: the window batch's offsets and hits (1 launch).
+//   launch_window_place: the window batch's offsets and its hits' places (1 launch).
+//   launch_window_z: per-hit z of the timeslice from its table (1 launch).
 //   launch_window_rows: triplet rows from window-batch indices to timeslice
 //     layer-group indices (1 launch).
 cudaError_t launch_window_ranges(const WinJob& w, cudaStream_t st);
-cudaError_t launch_window_gather(const WinJob& w, cudaStream_t st);
+cudaError_t launch_window_place(const WinJob& w, cudaStream_t st);
+cudaError_t launch_window_z(const WinJob& w, float* z, cudaStream_t st);
 cudaError_t launch_window_rows(const WinJob& w, const int64_t* trip_off, int32_t* triplets, cudaStream_t st);
 }  // namespace streamk
 constexpr int kLaunchesWindows = 6;

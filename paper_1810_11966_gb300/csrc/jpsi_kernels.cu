@@ -131,6 +131,7 @@ struct WarpTile {
     uint32_t pend[64];                    // triples: station << 27 | i << 18 | j << 9 | k
     uint8_t left[2][SmallCfg::LAYER_CAP]; // layer-local indices of the hits that the sieve leaves
     int32_t off[3 * kMaxStations + 1];    // the event's offsets
+    int32_t sh[kStream ? 3 * kMaxStations : 1];  // and shifts (free-streaming windows)
     int32_t count[kMaxStations];          // passing triplets per station
     float2 T[SmallCfg::TCAP];             // trigger triplet slopes
     union {
@@ -153,6 +154,7 @@ struct MediumTile {
     uint16_t left[3][MediumCfg::LAYER_CAP];
     int n_left[3];
     int32_t off[3 * kMaxStations + 1];
+    int32_t sh[kStream ? 3 * kMaxStations : 1];
     int32_t count[kMaxStations];
     int red[WARPS][3];                          // largest |slope|, largest and smallest 1/z (bit patterns)
     int s_gi, s_flag;
@@ -175,6 +177,7 @@ struct BlockSmem {
     alignas(4) uint16_t bst[3 * B::NC + 1];  // cell starts (cell counts while a layer is staged)
     LayerMeta meta[3];
     int32_t off[3 * kMaxStations + 1];
+    int32_t sh[kStream ? 3 * kMaxStations : 1];  // shifts (free-streaming windows)
     int32_t wsum[B::WARPS];
     int red_i[B::WARPS][2];
     int red_k[B::WARPS][7];
@@ -279,6 +282,18 @@ __device__ __forceinline__ void prefetch_hits_l2(const Job& j, int32_t h0, int32
     }
 }
 
+// The lines of station s of the event with these offsets (and shifts).
+__device__ __forceinline__ void prefetch_station(const Job& j, const int32_t* off, const int32_t* sh, int s, int lane) {
+    if (j.host_hits) return;
+    if constexpr (kStream) {
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+            prefetch_hits_l2(j, off[3 * s + l] + sh[3 * s + l], off[3 * s + l + 1] + sh[3 * s + l], lane);
+    } else {
+        prefetch_hits_l2(j, off[3 * s], off[3 * s + 3], lane);
+    }
+}
+
 __device__ __forceinline__ int station_of(int si, int trig) { return si == 0 ? trig : (si - 1 < trig ? si - 1 : si); }
 
 // Free-streaming windows: are the times a, b, c coincident (max t <=
@@ -294,6 +309,22 @@ __device__ __forceinline__ bool coincident3(float a, float b, float c, float dt,
 __device__ __forceinline__ bool partner_coincident(float pmin, float pmax, float2 T, float dt) {
     return pmax <= __fadd_rn(pmin, dt) && fmaxf(pmax, T.y) <= __fadd_rn(fminf(pmin, T.x), dt);
 }
+
+// Where a station's hits lie in the hit arrays: layer l at the station's own
+// offsets plus shift[l].  Events lie there in CSR order (no shift); the windows of a
+// timeslice are ranges of its layer groups, so their offsets only count hits.
+struct Shift3 {
+    int32_t a, b, c;
+    __device__ __forceinline__ int32_t of(int l) const { return l == 0 ? a : l == 1 ? b : c; }
+    // of the hit at place p of the station, whose layers 1 and 2 start at s1 and s2
+    __device__ __forceinline__ int32_t at(int p, int s1, int s2) const {
+        return !kStream ? 0 : p < s1 ? a : p < s2 ? b : c;
+    }
+};
+__device__ __forceinline__ Shift3 shift3(const int32_t* sh, int s) {
+    return kStream ? Shift3{sh[3 * s], sh[3 * s + 1], sh[3 * s + 2]} : Shift3{0, 0, 0};
+}
+constexpr int kShifts = kStream ? 3 * kMaxStations : 1;  // entries of an event's shifts in shared memory
 
 // Cell histogram of the layer being staged on a block tile, kept in place in
 // the layer's own cell-start array: two 16-bit counters per 32-bit word (a
@@ -972,14 +1003,15 @@ __device__ __forceinline__ StationBounds station_bounds(float rmax, float smax, 
 // odd coordinate: their slopes to P, (Inf, Inf) for a hit with a non-finite
 // coordinate (it passes no finite bound, and no fit in any case).  Returns 0, 1
 // (z <= 0) or 2 (a hit whose pruning bound is not finite).
-__device__ __forceinline__ int sieve_classify(const Job& j, float2* P, int lane, int32_t o0, int n, float& rmax,
-                                           float& smax) {
+__device__ __forceinline__ int sieve_classify(const Job& j, float2* P, int lane, int32_t o0, int s1, int s2, int n,
+                                              const Shift3& sh, float& rmax, float& smax) {
     bool zbad = false, wild = false;
     rmax = smax = 0.0f;
     __syncwarp();  // (the slopes written so far)
 #pragma unroll 1
     for (int p = lane; p < n; p += 32) {
-        const HitPrep h = hit_prep(__ldg(j.x + o0 + p), __ldg(j.y + o0 + p), __ldg(j.z + o0 + p), j.K);
+        const int32_t g = o0 + p + sh.at(p, s1, s2);
+        const HitPrep h = hit_prep(__ldg(j.x + g), __ldg(j.y + g), __ldg(j.z + g), j.K);
         zbad |= h.zbad;
         wild |= h.wild;
         const bool live = h.live & !h.wild;
@@ -1064,7 +1096,9 @@ __device__ __forceinline__ int light_fit(const Job& j, W& w, const uint32_t* pen
             ii = (en >> 18) & 511;
             jj = (en >> 9) & 511;
             kk = en & 511;
-            const int32_t h0 = w.off[3 * st] + ii, h1 = w.off[3 * st + 1] + jj, h2 = w.off[3 * st + 2] + kk;
+            const Shift3 sh = shift3(w.sh, st);
+            const int32_t h0 = w.off[3 * st] + ii + sh.a, h1 = w.off[3 * st + 1] + jj + sh.b,
+                          h2 = w.off[3 * st + 2] + kk + sh.c;
             const float xs[3] = {__ldg(j.x + h0), __ldg(j.x + h1), __ldg(j.x + h2)};
             const float ys[3] = {__ldg(j.y + h0), __ldg(j.y + h1), __ldg(j.y + h2)};
             const float zs[3] = {__ldg(j.z + h0), __ldg(j.z + h1), __ldg(j.z + h2)};
@@ -1123,14 +1157,20 @@ __device__ __forceinline__ int light_fit(const Job& j, W& w, const uint32_t* pen
 // the end of a layer, which read on into the hits behind it, would leave them.
 template <int R>
 __device__ __forceinline__ bool sieve_stage(const Job& j, WarpTile& w, int lane, int32_t o0, int n0, int n1, int n2,
-                                            float& rmax, float& smax) {
+                                            const Shift3& sh, float& rmax, float& smax) {
     const int nl[3] = {n0, n1, n2}, sl[3] = {0, n0, n0 + n1};
     rmax = smax = 0.0f;
-    if ((int64_t)o0 + sl[2] + 32 * R > j.n_hits) return false;
+    if constexpr (kStream) {
+        if ((int64_t)o0 + max(max(sh.a, sl[1] + sh.b), sl[2] + sh.c) + 32 * R > j.n_src) return false;
+    } else if ((int64_t)o0 + sl[2] + 32 * R > j.n_src) {
+        return false;
+    }
     float rmin = INFINITY;
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
-        const float *px = j.x + o0 + sl[l] + lane, *py = j.y + o0 + sl[l] + lane, *pz = j.z + o0 + sl[l] + lane;
+        const int32_t hs = kStream ? sh.of(l) : 0;
+        const float *px = j.x + o0 + sl[l] + hs + lane, *py = j.y + o0 + sl[l] + hs + lane,
+                    *pz = j.z + o0 + sl[l] + hs + lane;
         float x[R], y[R], z[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -1313,17 +1353,19 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
                                              int n1, int n2, int64_t e, int s, bool sink, bool all, StationBounds& sb,
                                              int& np) {
     const int most = max(max(n0, n1), n2);
+    const Shift3 sh = kStream ? Shift3{uniform(w.sh[3 * s]), uniform(w.sh[3 * s + 1]), uniform(w.sh[3 * s + 2])}
+                              : Shift3{0, 0, 0};
     float rmax, smax;
     bool ok;
     if (most <= 64)
-        ok = sieve_stage<2>(j, w, lane, o0, n0, n1, n2, rmax, smax);
+        ok = sieve_stage<2>(j, w, lane, o0, n0, n1, n2, sh, rmax, smax);
     else if (most <= 128)
-        ok = sieve_stage<4>(j, w, lane, o0, n0, n1, n2, rmax, smax);
+        ok = sieve_stage<4>(j, w, lane, o0, n0, n1, n2, sh, rmax, smax);
     else
-        ok = sieve_stage<6>(j, w, lane, o0, n0, n1, n2, rmax, smax);
+        ok = sieve_stage<6>(j, w, lane, o0, n0, n1, n2, sh, rmax, smax);
     sb = station_bounds(rmax, smax, j.K);
     if (!uniform(ok && sb.B < INFINITY)) {
-        const int st = uniform(sieve_classify(j, w.P, lane, o0, n0 + n1 + n2, rmax, smax));
+        const int st = uniform(sieve_classify(j, w.P, lane, o0, n0, n0 + n1, n0 + n1 + n2, sh, rmax, smax));
         if (st) return st;
         sb = station_bounds(rmax, smax, j.K);
     }
@@ -1349,14 +1391,14 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
 // pairs with 32 hits of layer 2 a step (P1 and P2).  Warp-uniform.
 template <class W>
 __device__ bool sieve_road(const Job& j, const W& w, int lane, const Cuts& c, const StationBounds& sb,
-                           int32_t o0, int n0, int n1, int n2, float mx, float my, float2 Tt) {
+                           int32_t o0, int n0, int n1, int n2, const Shift3& sh, float mx, float my, float2 Tt) {
     const int s1 = n0, s2 = n0 + n1, n = s2 + n2;
-    // the hits of places [p0, p0 + 32) of a layer ending at `end` that pass the tube
-    auto tube = [&](int p0, int end) {
+    // the hits of places [p0, p0 + 32) of a layer ending at `end` (hit index less place: g) that pass the tube
+    auto tube = [&](int p0, int end, int32_t g) {
         bool in = false;
         const float2 s = w.P[p0 + lane];
         if (p0 + lane < end && tube_ok(s.x, s.y, sb.b, mx, my)) {
-            const int32_t h = o0 + p0 + lane;
+            const int32_t h = g + p0 + lane;
             in = tube_pass(__ldg(j.x + h), __ldg(j.y + h), __ldg(j.z + h), mx, my, c);
         }
         return __ballot_sync(kFull, in);
@@ -1364,19 +1406,19 @@ __device__ bool sieve_road(const Job& j, const W& w, int lane, const Cuts& c, co
 #pragma unroll 1
     for (int i0 = 0; i0 < n0; i0 += 32) {
 #pragma unroll 1
-        for (unsigned mi = tube(i0, s1); mi; mi &= mi - 1) {
-            const int32_t h0 = o0 + i0 + __ffs(mi) - 1;
+        for (unsigned mi = tube(i0, s1, o0 + sh.a); mi; mi &= mi - 1) {
+            const int32_t h0 = o0 + sh.a + i0 + __ffs(mi) - 1;
 #pragma unroll 1
             for (int j0 = s1; j0 < s2; j0 += 32) {
 #pragma unroll 1
-                for (unsigned mj = tube(j0, s2); mj; mj &= mj - 1) {
-                    const int32_t h1 = o0 + j0 + __ffs(mj) - 1;
+                for (unsigned mj = tube(j0, s2, o0 + sh.b); mj; mj &= mj - 1) {
+                    const int32_t h1 = o0 + sh.b + j0 + __ffs(mj) - 1;
 #pragma unroll 1
                     for (int k0 = s2; k0 < n; k0 += 32) {
                         const float2 s = w.P[k0 + lane];
                         bool ok = false;
                         if (k0 + lane < n && tube_ok(s.x, s.y, sb.b, mx, my)) {
-                            const int32_t h2 = o0 + k0 + lane;
+                            const int32_t h2 = o0 + sh.c + k0 + lane;
                             const float xs[3] = {__ldg(j.x + h0), __ldg(j.x + h1), __ldg(j.x + h2)};
                             const float ys[3] = {__ldg(j.y + h0), __ldg(j.y + h1), __ldg(j.y + h2)};
                             const float zs[3] = {__ldg(j.z + h0), __ldg(j.z + h1), __ldg(j.z + h2)};
@@ -1425,7 +1467,10 @@ __device__ __forceinline__ int light_offsets(const Job& j, WarpTile& w, int lane
     const int rounds = S3 < 32 ? 1 : 2;
 #pragma unroll 1
     for (int q = 0; q < rounds; ++q)
-        if (lane + 32 * q <= S3) w.off[lane + 32 * q] = __ldg(base + lane + 32 * q);
+        if (lane + 32 * q <= S3) {
+            w.off[lane + 32 * q] = __ldg(base + lane + 32 * q);
+            if (kStream && lane + 32 * q < S3) w.sh[lane + 32 * q] = __ldg(j.shift + e * S3 + lane + 32 * q);
+        }
     __syncwarp();
     int code = 0;
     bool med = true;
@@ -1467,7 +1512,10 @@ __device__ void light_event_count(const Job& j, WarpTile& w, int lane, const Cut
         // the first station's lines start towards L2 now; each station then
         // prefetches the next (prefetching all of them evicted some lines
         // before use: 17 % more DRAM reads, against 4 % for one ahead)
-        if (!j.host_hits) prefetch_hits_l2(j, o0, w.off[3 * j.trig + 3], lane);
+        if (kStream)
+            prefetch_station(j, w.off, w.sh, j.trig, lane);
+        else if (!j.host_hits)
+            prefetch_hits_l2(j, o0, w.off[3 * j.trig + 3], lane);
         const bool sink = chain || j.distinct;  // the trigger triplets are kept: CHAIN slopes, candidates' hits
         int np = 0, nT = 0;
         if (lane < kMaxStations) w.count[lane] = 0;
@@ -1477,10 +1525,7 @@ __device__ void light_event_count(const Job& j, WarpTile& w, int lane, const Cut
             o0 = uniform(w.off[3 * s]);
             const int n0 = uniform(w.off[3 * s + 1]) - o0, n1 = uniform(w.off[3 * s + 2]) - o0 - n0,
                       n2 = uniform(w.off[3 * s + 3]) - o0 - n0 - n1;
-            if (si + 1 < nproc && !j.host_hits) {
-                const int sn = station_of(si + 1, j.trig);
-                prefetch_hits_l2(j, w.off[3 * sn], w.off[3 * sn + 3], lane);
-            }
+            if (si + 1 < nproc) prefetch_station(j, w.off, w.sh, station_of(si + 1, j.trig), lane);
             StationBounds sb;
             const int st = light_station<false>(j, w, lane, c, o0, n0, n1, n2, e, s, sink,
                                                 (sink && si == 0) || si + 1 == nproc, sb, np);
@@ -1500,7 +1545,7 @@ __device__ void light_event_count(const Job& j, WarpTile& w, int lane, const Cut
                 for (int ti = 0; ti < nT; ++ti) {  // (CHAIN only: PAPER has one station)
                     if (!w.alive[ti]) continue;
                     const float2 m = w.T[ti];
-                    const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, m.x, m.y,
+                    const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, shift3(w.sh, s), m.x, m.y,
                                                   kStream ? w.Tt[ti] : make_float2(0.f, 0.f));
                     if (!found && lane == 0) w.alive[ti] = 0;
                 }
@@ -1612,7 +1657,7 @@ __device__ int stage_station_block(const Job& j, BlockSmem<B>& sm, int s) {
     for (int l = 0; l < 3; ++l) {
         const int32_t b = sm.off[3 * s + l], e = sm.off[3 * s + l + 1];
         int nl = 0;
-        const int st = stage_layer_block(j, sm, l, b, e - b, pbase, nl);
+        const int st = stage_layer_block(j, sm, l, b + (kStream ? sm.sh[3 * s + l] : 0), e - b, pbase, nl);
         if (st) return st;
         pbase += nl;
     }
@@ -1622,7 +1667,10 @@ __device__ int stage_station_block(const Job& j, BlockSmem<B>& sm, int s) {
 template <class B>
 __device__ __forceinline__ void load_event_offsets(const Job& j, BlockSmem<B>& sm, int64_t e) {
     const int S3 = 3 * j.S;
-    for (int i = threadIdx.x; i <= S3; i += B::THREADS) sm.off[i] = j.off[e * S3 + i];
+    for (int i = threadIdx.x; i <= S3; i += B::THREADS) {
+        sm.off[i] = j.off[e * S3 + i];
+        if (kStream && i < S3) sm.sh[i] = j.shift[e * S3 + i];
+    }
     __syncthreads();
 }
 
@@ -1652,11 +1700,14 @@ constexpr int kGiPlain = -1;  // the one-launch form: the same block goes on unp
 template <class B>
 __device__ __forceinline__ void prefetch_station_block(const Job& j, const BlockSmem<B>& sm, int s) {
     if (j.host_hits) return;
-    const int32_t h0 = sm.off[3 * s], h1 = sm.off[3 * s + 3];
-    for (int32_t a = (h0 & ~31) + 32 * (int)threadIdx.x; a < h1; a += 32 * B::THREADS) {
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(j.x + a));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(j.y + a));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(j.z + a));
+    for (int l = 0; l < (kStream ? 3 : 1); ++l) {
+        const int32_t g = kStream ? sm.sh[3 * s + l] : 0;
+        const int32_t h0 = sm.off[3 * s + l] + g, h1 = sm.off[3 * s + (kStream ? l + 1 : 3)] + g;
+        for (int32_t a = (h0 & ~31) + 32 * (int)threadIdx.x; a < h1; a += 32 * B::THREADS) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(j.x + a));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(j.y + a));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(j.z + a));
+        }
     }
 }
 
@@ -1908,13 +1959,15 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
               n2 = uniform(w.off[3 * s + 3]) - o0 - n0 - n1, n = n0 + n1 + n2;
     const int s1 = n0, s2 = n0 + n1;
     constexpr int T = MediumTile::THREADS;
+    const Shift3 sh = shift3(w.sh, s);
     float smax = 0.0f, rmax = 0.0f, rmin = INFINITY;
     for (int p0 = 0; p0 < n; p0 += 4 * T) {
         float x[4], y[4], z[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             if (p0 + T * q < n) {  // block-uniform; threads past the end read the last hit again
-                const int32_t h = o0 + min(p0 + T * q + tid, n - 1);
+                const int p = min(p0 + T * q + tid, n - 1);
+                const int32_t h = o0 + p + sh.at(p, s1, s2);
                 x[q] = __ldg(j.x + h);
                 y[q] = __ldg(j.y + h);
                 z[q] = __ldg(j.z + h);
@@ -1955,7 +2008,8 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
         bool zbad = false, wild = false;
         smax = rmax = 0.0f;
         for (int p = tid; p < n; p += T) {
-            const HitPrep h = hit_prep(__ldg(j.x + o0 + p), __ldg(j.y + o0 + p), __ldg(j.z + o0 + p), j.K);
+            const int32_t g = o0 + p + sh.at(p, s1, s2);
+            const HitPrep h = hit_prep(__ldg(j.x + g), __ldg(j.y + g), __ldg(j.z + g), j.K);
             zbad |= h.zbad;
             wild |= h.wild;
             const bool live = h.live & !h.wild;
@@ -1999,7 +2053,10 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
     const int S = j.S;
     const bool chain = j.mode == 1 && S > 1;
     const int nproc = j.mode == 1 ? S : 1;
-    for (int i = tid; i <= 3 * S; i += MediumTile::THREADS) w.off[i] = __ldg(j.off + e * 3 * S + i);
+    for (int i = tid; i <= 3 * S; i += MediumTile::THREADS) {
+        w.off[i] = __ldg(j.off + e * 3 * S + i);
+        if (kStream && i < 3 * S) w.sh[i] = __ldg(j.shift + e * 3 * S + i);
+    }
     if (tid < kMaxStations) w.count[tid] = 0;
     __syncthreads();
     int np = 0, nT = 0;
@@ -2009,12 +2066,9 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
         const int s = station_of(si, j.trig);
         const int cnt = EMIT ? uniform(j.unit_counts[e * S + s]) : 0;
         if (EMIT && cnt == 0) continue;
-        if (!j.host_hits && wp == 0) {  // the next station's lines start towards L2
-            if (si == 0) prefetch_hits_l2(j, w.off[3 * s], w.off[3 * s + 3], lane);
-            if (si + 1 < nproc) {
-                const int sn = station_of(si + 1, j.trig);
-                prefetch_hits_l2(j, w.off[3 * sn], w.off[3 * sn + 3], lane);
-            }
+        if (wp == 0) {  // the next station's lines start towards L2
+            if (si == 0) prefetch_station(j, w.off, w.sh, s, lane);
+            if (si + 1 < nproc) prefetch_station(j, w.off, w.sh, station_of(si + 1, j.trig), lane);
         }
         StationBounds sb;
         const int st = medium_station<EMIT>(j, w, c, e, s, sink, EMIT || (sink && si == 0) || si + 1 == nproc, sb, np);
@@ -2049,7 +2103,7 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
             for (int ti = wp; ti < nT; ti += MediumTile::WARPS) {  // (CHAIN only: PAPER has one station)
                 if (!w.alive[ti]) continue;
                 const float2 m = w.T[ti];
-                const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, m.x, m.y,
+                const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, shift3(w.sh, s), m.x, m.y,
                                               kStream ? w.Tt[ti] : make_float2(0.f, 0.f));
                 __syncwarp();
                 if (!found && lane == 0) w.alive[ti] = 0;
@@ -2282,18 +2336,20 @@ __device__ __forceinline__ GHit ghit(const Job& j, int64_t h) {
 }
 
 // Brute-force P2 search over every hit of every other station.
-__device__ bool road_global(const Job& j, const int32_t* soff, const Cuts& c, float mx, float my, float2 Tt) {
+__device__ bool road_global(const Job& j, const int32_t* soff, const int32_t* sh, const Cuts& c, float mx, float my,
+                            float2 Tt) {
     for (int s = 0; s < j.S; ++s) {
         if (s == j.trig) continue;
         const int32_t* o = soff + 3 * s;
+        const Shift3 g = shift3(sh, s);
         bool found = false;
-        for (int32_t h0 = o[0]; h0 < o[1] && !found; ++h0) {
+        for (int32_t h0 = o[0] + g.a; h0 < o[1] + g.a && !found; ++h0) {
             const float x0 = __ldg(j.x + h0), y0 = __ldg(j.y + h0), z0 = __ldg(j.z + h0);
             if (!tube_pass(x0, y0, z0, mx, my, c)) continue;
-            for (int32_t h1 = o[1]; h1 < o[2] && !found; ++h1) {
+            for (int32_t h1 = o[1] + g.b; h1 < o[2] + g.b && !found; ++h1) {
                 const float x1 = __ldg(j.x + h1), y1 = __ldg(j.y + h1), z1 = __ldg(j.z + h1);
                 if (!tube_pass(x1, y1, z1, mx, my, c)) continue;
-                for (int32_t h2 = o[2]; h2 < o[3] && !found; ++h2) {
+                for (int32_t h2 = o[2] + g.c; h2 < o[3] + g.c && !found; ++h2) {
                     const float xs[3] = {x0, x1, __ldg(j.x + h2)};
                     const float ys[3] = {y0, y1, __ldg(j.y + h2)};
                     const float zs[3] = {z0, z1, __ldg(j.z + h2)};
@@ -2316,6 +2372,7 @@ __device__ bool road_global(const Job& j, const int32_t* soff, const Cuts& c, fl
 // Shared scratch of the unpruned search of one event (from the caller).
 struct GenShared {
     int32_t* soff;  // [3 * kMaxStations + 1] the event's offsets
+    int32_t* sh;    // [kShifts] and shifts (free-streaming windows)
     int* s_count;
     int* s_cand;
     int* s_bad;
@@ -2350,7 +2407,7 @@ __device__ void generic_candidates(const Job& j, const int32_t* soff, const Cuts
             const float xs[3] = {hi.x, hj.x, hk.x}, ys[3] = {hi.y, hj.y, hk.y}, zs[3] = {hi.z, hj.z, hk.z};
             float mx, my;
             if (!fit_pass(xs, ys, zs, c, mx, my)) continue;
-            if (chain && !road_global(j, soff, c, mx, my, make_float2(0.f, 0.f))) continue;  // (no streams here)
+            if (chain && !road_global(j, soff, nullptr, c, mx, my, make_float2(0.f, 0.f))) continue;  // (no streams here)
             const int r = atomicAdd(s_rank, 1);
             if (r < cap) out[r] = pack_ijk((int)i, (int)jx, (int)k);
         }
@@ -2369,7 +2426,10 @@ __device__ void generic_event(const Job& j, int64_t e, const GenShared& g) {
     const int nproc = j.mode == 1 ? S : 1;
     int32_t* soff = g.soff;
     __syncthreads();  // earlier users of the shared scratch are done
-    for (int i = threadIdx.x; i <= S3; i += blockDim.x) soff[i] = j.off[e * S3 + i];
+    for (int i = threadIdx.x; i <= S3; i += blockDim.x) {
+        soff[i] = j.off[e * S3 + i];
+        if (kStream && i < S3) g.sh[i] = j.shift[e * S3 + i];
+    }
     if (threadIdx.x == 0) *g.s_cand = 0;
     __syncthreads();
     int trig_count = 0;
@@ -2378,6 +2438,7 @@ __device__ void generic_event(const Job& j, int64_t e, const GenShared& g) {
         const int s = station_of(si, j.trig);
         const int64_t u = e * S + s;
         const int32_t* o = soff + 3 * s;
+        const Shift3 b = shift3(g.sh, s);
         if (EMIT && j.unit_counts[u] == 0) continue;
         if (threadIdx.x == 0) {
             *g.s_count = 0;
@@ -2385,8 +2446,8 @@ __device__ void generic_event(const Job& j, int64_t e, const GenShared& g) {
         }
         __syncthreads();
         if (!EMIT) {
-            for (int32_t h = o[0] + threadIdx.x; h < o[3]; h += blockDim.x)
-                if (__ldg(j.z + h) <= 0.0f) *g.s_bad = 1;
+            for (int32_t p = o[0] + threadIdx.x; p < o[3]; p += blockDim.x)
+                if (__ldg(j.z + p + b.at(p, o[1], o[2])) <= 0.0f) *g.s_bad = 1;
             __syncthreads();
             if (*g.s_bad) {
                 if (threadIdx.x == 0) {
@@ -2405,12 +2466,12 @@ __device__ void generic_event(const Job& j, int64_t e, const GenShared& g) {
         const bool collect = !EMIT && chain && s == j.trig;
         for (int64_t p = threadIdx.x; p < npairs; p += blockDim.x) {
             const int64_t i = p / n1, jx = p - i * n1;
-            const GHit hi = ghit(j, o[0] + i), hj = ghit(j, o[1] + jx);
+            const GHit hi = ghit(j, o[0] + b.a + i), hj = ghit(j, o[1] + b.b + jx);
             if (!hi.p.live || !hj.p.live) continue;
             if (!hi.p.wild && !hj.p.wild && !pair_ok(hi.p.sx, hi.p.sy, hj.p.sx, hj.p.sy, __fadd_rn(hi.p.b, hj.p.b)))
                 continue;
             for (int64_t k = 0; k < n2; ++k) {
-                const GHit hk = ghit(j, o[2] + k);
+                const GHit hk = ghit(j, o[2] + b.c + k);
                 if (!hk.p.live) continue;
                 if (!hk.p.wild) {
                     if (!hi.p.wild && !pair_ok(hi.p.sx, hi.p.sy, hk.p.sx, hk.p.sy, __fadd_rn(hi.p.b, hk.p.b)))
@@ -2423,7 +2484,7 @@ __device__ void generic_event(const Job& j, int64_t e, const GenShared& g) {
                 if (!fit_pass(xs, ys, zs, c, mx, my)) continue;
                 float2 Tt = make_float2(0.f, 0.f);
                 if constexpr (kStream) {  // coincident and owned by this window
-                    const bool co = coincident3(__ldg(j.t + o[0] + i), __ldg(j.t + o[1] + jx), __ldg(j.t + o[2] + k), j.dt,
+                    const bool co = coincident3(__ldg(j.t + o[0] + b.a + i), __ldg(j.t + o[1] + b.b + jx), __ldg(j.t + o[2] + b.c + k), j.dt,
                                                 Tt.x, Tt.y);
                     if (!(co && Tt.x >= __ldg(j.wb + e) && Tt.x < __ldg(j.wb + e + 1))) continue;
                 }
@@ -2433,14 +2494,14 @@ __device__ void generic_event(const Job& j, int64_t e, const GenShared& g) {
                     if (i >= kPackLimit || jx >= kPackLimit || k >= kPackLimit) {
                         atomicOr(&j.ctrl->status, kStNoScratch);
                     } else {
-                        const unsigned long long b = atomicAdd(&j.ctrl->scratch_n, 1ull);
-                        if (b < (unsigned long long)j.tscr_cap) {
+                        const unsigned long long at = atomicAdd(&j.ctrl->scratch_n, 1ull);
+                        if (at < (unsigned long long)j.tscr_cap) {
                             TripEntry te;
                             te.unit = (int32_t)u;
                             te.rank = rk;
                             te.ijk = (unsigned long long)i | ((unsigned long long)jx << 20) |
                                      ((unsigned long long)k << 40) | ((unsigned long long)kClsGeneric << kTagShift);
-                            j.tscr[b] = te;
+                            j.tscr[at] = te;
                         }
                     }
                 }
@@ -2454,7 +2515,7 @@ __device__ void generic_event(const Job& j, int64_t e, const GenShared& g) {
                         r[2] = (int32_t)k;
                     }
                 }
-                if (collect && road_global(j, soff, c, mx, my, Tt)) atomicAdd(g.s_cand, 1);
+                if (collect && road_global(j, soff, g.sh, c, mx, my, Tt)) atomicAdd(g.s_cand, 1);
             }
         }
         if (!EMIT && !j.tscr && local) atomicAdd(g.s_count, local);
@@ -2503,6 +2564,7 @@ __device__ void generic_event(const Job& j, int64_t e, const GenShared& g) {
 template <bool EMIT>
 __global__ void __launch_bounds__(kGenThreads) k_generic(const __grid_constant__ Job j) {
     __shared__ int32_t soff[3 * kMaxStations + 1];
+    __shared__ int32_t sh[kShifts];
     __shared__ int s_gi, s_count, s_cand, s_bad;
     __shared__ unsigned long long s_pool;
     chain_wait();
@@ -2514,7 +2576,7 @@ __global__ void __launch_bounds__(kGenThreads) k_generic(const __grid_constant__
         if (gi >= n_gen) break;
         const int64_t e = j.glist[gi];
         if (!EMIT || j.ev_class[e] == kClsGeneric)
-            generic_event<EMIT>(j, e, GenShared{soff, &s_count, &s_cand, &s_bad, &s_pool});
+            generic_event<EMIT>(j, e, GenShared{soff, sh, &s_count, &s_cand, &s_bad, &s_pool});
         __syncthreads();
     }
     chain_next();
@@ -2660,7 +2722,7 @@ __global__ void __launch_bounds__(kHThreads, 3) k_plain_block(const __grid_const
     const uint8_t cls = j.ev_class[e];
     bool generic = cls == kClsGeneric;
     if (cls == kClsHeavy) generic = plain_block_event<EMIT>(j, ps, e);
-    if (generic) generic_event<EMIT>(j, e, GenShared{ps.h.off, &ps.h.s_rank, &ps.h.s_cand, &ps.h.s_next, &ps.h.s_pool});
+    if (generic) generic_event<EMIT>(j, e, GenShared{ps.h.off, ps.h.sh, &ps.h.s_rank, &ps.h.s_cand, &ps.h.s_next, &ps.h.s_pool});
 }
 
 // -------------------------------------------------------- accept bits
@@ -3079,9 +3141,12 @@ cudaError_t launch_emit_phase(const Job& job, int64_t n_events, const LaunchCfg&
 // (the trigger station: [b_k, fl32(b_k+1 + dt)], which holds every triplet
 // owned by the window; the other stations of CHAIN mode from a margin below
 // b_k - dt to the same end, which holds every partner that can be coincident
-// with such a triplet).  The selection kernels of this build then apply the
-// time tests themselves; the rows they write index the window batch and are
-// moved back to timeslice group indices at the end.
+// with such a triplet).  The batch is only offsets and shifts: the selection
+// kernels of this build read the hits where they lie in the timeslice (a copy
+// of the ranges took 0.96 ms of a 10^5-collision timeslice, 3.53 ms, and 16
+// bytes per hit of the ranges) and apply the time tests themselves; the rows
+// they write index the window batch and are moved back to timeslice group
+// indices at the end.
 
 // Last group q < S3 with so[q] <= h (so: the 3S+1 offsets, non-decreasing).
 __device__ __forceinline__ int group_of(const int32_t* so, int S3, int64_t h) {
@@ -3195,58 +3260,29 @@ __global__ void __launch_bounds__(256) k_win_ranges(const __grid_constant__ WinJ
     }
 }
 
-// The window batch: its offsets (from the scan) and its hits, one warp per
-// (window, group) range.  Bound by memory (each hit of a range is read and
-// written once: 32 bytes): four rounds of a range, 16 loads per lane, are in
-// flight before the first store, and the next range's place is read ahead (144 M
-// window hits of 120 M: 1270 -> 964 us, 5.0 TB/s of DRAM traffic).
-__global__ void __launch_bounds__(256) k_win_gather(const __grid_constant__ WinJob w) {
-    const int S3 = 3 * w.S;
-    const int64_t n = w.K * S3;
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int64_t dst = 0, src = 0;
-    int cnt = 0;
-    auto place = [&](int64_t i) {
-        if (i < n) {
-            dst = w.woff[i];
-            src = w.wlo[i];
-            cnt = w.wcnt[i];
-        }
-    };
-    place(q);
-    constexpr int Q = 4;
-    for (; q < n; q += nwarps) {
-        const int64_t d = dst, s = src;
-        const int m = cnt;
-        place(q + nwarps);
-        if (lane == 0) w.off_out[q] = (int32_t)d;
-        if (m == 0) continue;  // (a timeslice without hits may come without z and z_layer)
-        const float zl = w.z ? 0.f : __ldg(w.z_layer + (int)(q % S3));
-        for (int i0 = 0; i0 < m; i0 += 32 * Q) {
-            float x[Q], y[Q], z[Q], t[Q];
-#pragma unroll
-            for (int r = 0; r < Q; ++r) {
-                const int64_t h = s + min(i0 + 32 * r + lane, m - 1);
-                x[r] = __ldg(w.x + h);
-                y[r] = __ldg(w.y + h);
-                z[r] = w.z ? __ldg(w.z + h) : zl;
-                t[r] = __ldg(w.t + h);
-            }
-#pragma unroll
-            for (int r = 0; r < Q; ++r) {
-                const int i = i0 + 32 * r + lane;
-                if (i < m) {
-                    w.xo[d + i] = x[r];
-                    w.yo[d + i] = y[r];
-                    w.zo[d + i] = z[r];
-                    w.to[d + i] = t[r];
-                }
-            }
-        }
+// The window batch: its offsets (from the scan), and how far its hits lie from
+// there in the timeslice.  The selection reads them where they are.
+__global__ void __launch_bounds__(256) k_win_place(const __grid_constant__ WinJob w) {
+    const int64_t n = w.K * 3 * w.S, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q <= n; q += stride) {
+        const int64_t at = w.woff[q];
+        w.off_out[q] = (int32_t)at;
+        if (q < n) w.shift[q] = (int32_t)(w.wlo[q] - at);
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) w.off_out[n] = (int32_t)w.woff[n];
+}
+
+// Per-hit z of the timeslice from the per-group table.
+__global__ void __launch_bounds__(256) k_win_fill_z(const __grid_constant__ WinJob w, float* __restrict__ z) {
+    __shared__ int32_t so[3 * kMaxStations + 1];
+    const int S3 = 3 * w.S;
+    for (int i = threadIdx.x; i <= S3; i += blockDim.x) so[i] = w.off[i];
+    __syncthreads();
+    for (int g = 0; g < S3; ++g) {
+        const float v = __ldg(w.z_layer + g);
+        for (int64_t h = so[g] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < so[g + 1];
+             h += (int64_t)gridDim.x * blockDim.x)
+            z[h] = v;
+    }
 }
 
 // Triplet rows of unit (k, s): window-batch layer indices plus the start of
@@ -3295,8 +3331,13 @@ cudaError_t launch_window_ranges(const WinJob& w, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_window_gather(const WinJob& w, cudaStream_t st) {
-    k_win_gather<<<win_grid(w.K * 3 * w.S * 32, w.n_sm), 256, 0, st>>>(w);
+cudaError_t launch_window_place(const WinJob& w, cudaStream_t st) {
+    k_win_place<<<win_grid(w.K * 3 * w.S + 1, w.n_sm), 256, 0, st>>>(w);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_window_z(const WinJob& w, float* z, cudaStream_t st) {
+    k_win_fill_z<<<win_grid(w.n_hits / (3 * w.S) + 1, w.n_sm), 256, 0, st>>>(w, z);
     return cudaGetLastError();
 }
 
@@ -3377,7 +3418,7 @@ extern "C" jpsi_status jpsi_select_noalloc(const jpsi_params* p, const jpsi_batc
     j.z = b->z;
     j.off = b->offsets;
     j.n_events = b->n_events;
-    j.n_hits = b->n_hits;
+    j.n_hits = j.n_src = b->n_hits;
     j.ev_begin = 0;
     j.ev_count = b->n_events;
     j.S = p->n_stations;
