@@ -511,12 +511,12 @@ def run_free_stream(args, w, dev, jp, torch):
     ms_p = tot_p / len(per_p)
     runs = max(tm_b.runs, 1)
     win_ms = tm_b.window_ms / runs
-    # the event-building phase moves at least: t and z of every hit (checks),
-    # x, y, z, t of every window-batch hit read and written once, the ranges
-    # (first hit, size, offset in 64 and 32 bits), and each triplet row read
-    # and written once by the mapping back
+    # the event-building phase moves at least: t and z of every hit (checks; the
+    # hits themselves stay where they are), the ranges (first hit, size, offset in
+    # 64 and 32 bits, shift), and each triplet row read and written once by the
+    # mapping back
     built = jp_window_hits(ts, p)
-    alg = 8 * n_hits + 32 * built + K * 3 * S * (4 + 4 + 8 + 4) + 24 * cap
+    alg = 8 * n_hits + K * 3 * S * (4 + 4 + 8 + 4 + 4) + 24 * cap
     peak, peak_kind = measured_peaks()
     achieved = alg / (win_ms / 1000.0) / 1e9
     per_sorted = sorted(per_b)
@@ -535,7 +535,7 @@ def run_free_stream(args, w, dev, jp, torch):
         "latency_ms": {"p50": per_sorted[len(per_sorted) // 2], "max": per_sorted[-1]},
         "phases_ms": {"event_building": win_ms, "light_count": tm_b.light_ms / runs,
                       "count_rest": tm_b.count_rest_ms / runs, "emit": tm_b.emit_ms / runs},
-        "roofline": {"bound": "hbm", "kernel": "event building (k_win_check, k_win_ranges, scan, k_win_gather, "
+        "roofline": {"bound": "hbm", "kernel": "event building (k_win_check, k_win_ranges, scan, k_win_place, "
                      "k_win_rows)", "achieved": achieved, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None, "algorithmic_bytes": alg},
         "e2e": {"value": n_coll / e2e_mean, "unit": "collisions/s", "h2d_bytes_per_step": h2d,
@@ -551,7 +551,7 @@ def run_free_stream(args, w, dev, jp, torch):
 
 
 def jp_window_hits(ts, p):
-    """Hits of the window batch (the ranges the library gathers), counted on
+    """Hits of the window batch (the ranges the library selects from), counted on
     the host from the timeslice: the trigger station's [b_k, fl32(b_k+1 + dt)],
     the other stations (CHAIN) from just below b_k - dt to the same end."""
     t, off, b = ts["t"], ts["offsets"], ts["bounds"].astype(np.float32)

@@ -1027,6 +1027,17 @@ __device__ __forceinline__ int sieve_classify(const Job& j, float2* P, int lane,
     return __any_sync(kFull, zbad) ? 1 : __any_sync(kFull, wild) ? 2 : 0;
 }
 
+// Is a station of the medium path too dense for the sieve?  It lets a hit through
+// when another layer has one within about 1.5 B of it in both slopes, so with n
+// hits per layer n B^2 says how selective it is (the slopes of a detector fill
+// about the same area).  Beyond kDense the event goes on to the block tile: 3 000
+// events of n = 250 and a 1 cm window (0.078 at z = 120 cm) 599 us, 818 with the sieve
+// (a medium cell-sorted tile took 390); 15 000 events of n = 150, 1 cm (0.047): the
+// sieve 853 us, the block tile 1 588 (cells 635).  Below, the sieve is the best of the
+// three (n = 300, 0.5 cm, 0.021: 269 us, cells 301).
+constexpr float kDense = 0.06f;
+__device__ __forceinline__ bool too_dense(int most, float B) { return (float)most * B * B > kDense; }
+
 // The cell of a slope: the nearest integer of s * inv, modulo the map's size
 // when it is used.  |s * inv| <= 4096, so the sum with 1.5 * 2^23 holds that
 // integer in its low mantissa bits (one rounding).  Hits of one passing
@@ -1160,6 +1171,9 @@ __device__ __forceinline__ bool sieve_stage(const Job& j, WarpTile& w, int lane,
                                             const Shift3& sh, float& rmax, float& smax) {
     const int nl[3] = {n0, n1, n2}, sl[3] = {0, n0, n0 + n1};
     rmax = smax = 0.0f;
+    // hits read over the host link: none that is not needed (200 000 events of 20
+    // hits per layer, PAPER: 1.69 ms with full rounds, 1.11 without)
+    if (j.host_hits) return false;
     if constexpr (kStream) {
         if ((int64_t)o0 + max(max(sh.a, sl[1] + sh.b), sl[2] + sh.c) + 32 * R > j.n_src) return false;
     } else if ((int64_t)o0 + sl[2] + 32 * R > j.n_src) {
@@ -1947,8 +1961,9 @@ __device__ __forceinline__ void medium_pass(const Job& j, MediumTile& w, float i
 
 // Stages station s of the event in w.off and finds its triples (see
 // sieve_layers; a third map leaves fewer hits of layer 1 when layer 2 has more
-// than kFilterMin).  Returns 0, 1 for a hit with z <= 0 or 2 for one whose
-// pruning bound is not finite; block-uniform, all threads call it.
+// than kFilterMin).  Returns 0, 1 for a hit with z <= 0, 2 for one whose pruning
+// bound is not finite or 3 for a station too dense for the sieve; block-uniform,
+// all threads call it.
 constexpr int kFilterMin = 8;
 template <bool EMIT>
 __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const Cuts& c, int64_t e, int s, bool sink,
@@ -2023,6 +2038,7 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
         if (uniform(__syncthreads_or(wild))) return 2;
         reduce();
     }
+    if (!EMIT && uniform(too_dense(max(max(n0, n1), n2), sb.B))) return 3;
     for (int p0 = 0; p0 < n1; p0 += T) {
         const SieveBit b = medium_bit(w.P[s1 + p0 + tid], sb.inv);
         if (p0 + tid < n1) atomicOr(&ma[b.word], b.bit);
@@ -2083,7 +2099,7 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
                     atomicOr(&j.ctrl->status, kStInvalid);
                     j.ev_class[e] = kClsInvalid;
                 } else {
-                    push_event(j, e, kClsGeneric);
+                    push_event(j, e, st == 2 ? kClsGeneric : kClsHeavy);
                 }
             }
             return;
