@@ -1497,12 +1497,15 @@ __device__ __forceinline__ int light_offsets(const Job& j, WarpTile& w, int lane
             if (l == S3) {
                 if ((int64_t)a > j.n_hits || (e == j.n_events - 1 && (int64_t)a != j.n_hits)) code = 2;
             } else {
+                // compared, not subtracted: 2^31 - 1 and -2 differ by 2^31 - 1
+                // in 32 bits.  (The sizes are right when no lane says 2.)
                 const int s = l / 3;
-                const int32_t d1 = w.off[l + 1] - a, d3 = l == 3 * s ? w.off[l + 3] - a : 0;
-                if (d1 < 0) code = 2;
+                if (w.off[l + 1] < a) code = 2;
+                const uint32_t d1 = (uint32_t)w.off[l + 1] - (uint32_t)a,
+                               d3 = l == 3 * s ? (uint32_t)w.off[l + 3] - (uint32_t)a : 0u;
                 if (j.mode == 1 || s == j.trig) {
-                    if (d1 > j.cap_small || d3 > SmallCfg::HCAP) code = max(code, 1);
-                    if (d1 > j.cap_medium || d3 > MediumCfg::HCAP) med = false;
+                    if (d1 > (uint32_t)j.cap_small || d3 > (uint32_t)SmallCfg::HCAP) code = max(code, 1);
+                    if (d1 > (uint32_t)j.cap_medium || d3 > (uint32_t)MediumCfg::HCAP) med = false;
                 }
             }
         }
