@@ -1027,17 +1027,6 @@ __device__ __forceinline__ int sieve_classify(const Job& j, float2* P, int lane,
     return __any_sync(kFull, zbad) ? 1 : __any_sync(kFull, wild) ? 2 : 0;
 }
 
-// Is a station of the medium path too dense for the sieve?  It lets a hit through
-// when another layer has one within about 1.5 B of it in both slopes, so with n
-// hits per layer n B^2 says how selective it is (the slopes of a detector fill
-// about the same area).  Beyond kDense the event goes on to the block tile: 3 000
-// events of n = 250 and a 1 cm window (0.078 at z = 120 cm) 599 us, 818 with the sieve
-// (a medium cell-sorted tile took 390); 15 000 events of n = 150, 1 cm (0.047): the
-// sieve 853 us, the block tile 1 588 (cells 635).  Below, the sieve is the best of the
-// three (n = 300, 0.5 cm, 0.021: 269 us, cells 301).
-constexpr float kDense = 0.06f;
-__device__ __forceinline__ bool too_dense(int most, float B) { return (float)most * B * B > kDense; }
-
 // The cell of a slope: the nearest integer of s * inv, modulo the map's size
 // when it is used.  |s * inv| <= 4096, so the sum with 1.5 * 2^23 holds that
 // integer in its low mantissa bits (one rounding).  Hits of one passing
@@ -1282,6 +1271,147 @@ __device__ __forceinline__ void sieve_layers(const Job& j, WarpTile& w, int lane
     __syncwarp();
 }
 
+// Crowded stations (wide windows: the maps let most hits through).  Trying every
+// hit that is left with every other grows with the square of the hits, so there
+// layers 0 and 1 are put in the order of their cells' rows, and a hit looks at
+// three rows of them.  The lists take the maps' memory, which is free by then.
+// Bound by instruction issue: two passes over the hits make the lists, then a step
+// of a walk is two loads, the pair test and a vote for 32 hits.
+//   L: the type of the indices; MAX: hits per layer; Q: pair queues (one per warp).
+constexpr int kRowQueue = 64;
+template <class L, int MAX, int Q>
+struct RowLists {
+    uint32_t end[2][kMapRows];  // where each row's hits end (layer 0, layer 1)
+    L order[2][MAX];            // layer-local indices by row
+    uint32_t queue[Q][kRowQueue];  // pairs: j << 9 | k
+};
+
+// The row of a hit's cell.
+__device__ __forceinline__ int sieve_row(float2 s, float inv) { return sieve_cell(s.y, inv) & (kMapRows - 1); }
+
+// Fills the lists from m0 hits of layer 0 (l0) and m1 of layer 1 (l1, or all of
+// them when it is null), whose slopes start at places 0 and s1.  All T threads
+// (a warp or a block) call it.
+template <int T, class R, class L>
+__device__ __forceinline__ void row_lists(R& r, const float2* P, int tid, float inv, const L* l0, int m0, const L* l1,
+                                          int m1, int s1) {
+    auto sync = [] {
+        if constexpr (T == 32)
+            __syncwarp();
+        else
+            __syncthreads();
+    };
+    const int lane = tid & 31;
+    sync();  // the maps are done with
+    for (int q = tid; q < 2 * kMapRows; q += T) r.end[0][q] = 0u;
+    sync();
+#pragma unroll 1
+    for (int q = tid; q < m0 + m1; q += T) {
+        const bool a = q < m0;
+        const int h = a ? l0[q] : l1 ? l1[q - m0] : q - m0;
+        atomicAdd(&r.end[a ? 0 : 1][sieve_row(P[a ? h : s1 + h], inv)], 1u);
+    }
+    sync();
+    // rows' starts (four rows a lane); placing the hits turns them into ends
+    if (tid < 32) {
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            uint4* p = reinterpret_cast<uint4*>(r.end[l]) + lane;
+            const uint4 c = *p;
+            const uint32_t b = (uint32_t)warp_incl_scan((int)(c.x + c.y + c.z + c.w), lane) - (c.x + c.y + c.z + c.w);
+            *p = make_uint4(b, b + c.x, b + c.x + c.y, b + c.x + c.y + c.z);
+        }
+    }
+    sync();
+#pragma unroll 1
+    for (int q = tid; q < m0 + m1; q += T) {
+        const bool a = q < m0;
+        const int h = a ? l0[q] : l1 ? l1[q - m0] : q - m0;
+        r.order[a ? 0 : 1][atomicAdd(&r.end[a ? 0 : 1][sieve_row(P[a ? h : s1 + h], inv)], 1u)] = (L)h;
+    }
+    sync();
+}
+
+// The hits of a row and of the rows beside it (a ring): up to two runs of the order.
+struct RowRuns {
+    int a, n, a2, len;  // the first run [a, a + n), the second from a2; hits of both
+    __device__ __forceinline__ int at(int t) const { return t < n ? a + t : a2 + (t - n); }
+};
+__device__ __forceinline__ RowRuns row_runs(const uint32_t* end, int row) {
+    constexpr int kLast = kMapRows - 1;
+    RowRuns w;
+    w.a = row > 1 ? (int)end[row - 2] : 0;
+    w.n = (int)end[min(row + 1, kLast)] - w.a;
+    w.a2 = row == 0 ? (int)end[kLast - 1] : 0;
+    w.len = w.n + (row == 0 ? (int)(end[kLast] - end[kLast - 1]) : row == kLast ? (int)end[0] : 0);
+    return w;
+}
+
+// The triples of a crowded station (see sieve_triples, whose pending triples and
+// fits they share): 32 hits of l2 at a time (k_first + k_step (32 b + lane)) look
+// for partners in their rows of layer 1, and 32 of the pairs found for partners in
+// theirs of layer 0, each lane walking its own runs.
+template <bool EMIT, class W, class R, class L>
+__device__ __forceinline__ int row_triples(const Job& j, W& w, uint32_t* pend, const R& r, uint32_t* queue, int lane,
+                                            const Cuts& c, float B, float inv, int64_t e, int s, int s1, int s2,
+                                            const L* l2, int m2, int k_first, int k_step, bool sink, int np) {
+    const uint32_t lt = (1u << lane) - 1u;
+    // what lives on across a fit: the hits of l2 from kb on are due, from step t of
+    // their runs; qn pairs wait; behind them dn are looking for partners, from step u
+    int kb = k_first, t = 0, qn = 0, dn = 0, u = 0;
+#pragma unroll 1
+    for (;;) {
+        if (dn == 0) {
+#pragma unroll 1
+            while (qn < 32 && kb < m2) {
+                const int k = kb + k_step * lane;
+                const int hk = l2[min(k, m2 - 1)];
+                const float2 Pk = w.P[s2 + hk];
+                const RowRuns rk = row_runs(r.end[1], sieve_row(Pk, inv));
+                const int len = k < m2 ? rk.len : 0, steps = __reduce_max_sync(kFull, len);
+#pragma unroll 1
+                for (; t < steps && qn < 32; ++t) {
+                    const bool in = t < len;
+                    const int hj = r.order[1][in ? rk.at(t) : 0];
+                    const float2 Pj = w.P[s1 + hj];
+                    const bool pass = in & pair_ok(Pj.x, Pj.y, Pk.x, Pk.y, B);
+                    const unsigned mask = __ballot_sync(kFull, pass);
+                    const int at = qn + __popc(mask & lt);
+                    if (pass && JPSI_IN(j.ctrl, at < kRowQueue)) queue[at] = (uint32_t)hj << 9 | (uint32_t)hk;
+                    qn += __popc(mask);
+                }
+                if (t >= steps) {
+                    kb += 32 * k_step;
+                    t = 0;
+                }
+            }
+            if (qn == 0) break;
+            dn = min(qn, 32);
+            qn -= dn;
+            u = 0;
+            __syncwarp();
+        }
+        const uint32_t en = queue[qn + min(lane, dn - 1)];
+        const float2 Qj = w.P[s1 + (int)(en >> 9)], Qk = w.P[s2 + (int)(en & 511u)];
+        const RowRuns ri = row_runs(r.end[0], sieve_row(Qj, inv));
+        const int len = lane < dn ? ri.len : 0, steps = __reduce_max_sync(kFull, len);
+#pragma unroll 1
+        for (; u < steps && np <= 32; ++u) {
+            const bool in = u < len;
+            const int hi = r.order[0][in ? ri.at(u) : 0];
+            const float2 Pi = w.P[hi];
+            const bool cand = in & pair_ok(Pi.x, Pi.y, Qj.x, Qj.y, B) & pair_ok(Pi.x, Pi.y, Qk.x, Qk.y, B);
+            const unsigned mask = __ballot_sync(kFull, cand);
+            const int at = np + __popc(mask & lt);
+            if (cand && JPSI_IN(j.ctrl, at < 64)) pend[at] = (uint32_t)s << 27 | (uint32_t)hi << 18 | en;
+            np += __popc(mask);
+        }
+        if (u >= steps) dn = 0;
+        np = light_fit<EMIT>(j, w, pend, lane, c, e, sink, uniform(np), 32);
+    }
+    return uniform(np);
+}
+
 // The triples whose pairs are all close enough, among the hits that the sieve
 // left of layers 0 (l0[0, m0)) and 2 (l2[0, m2)) and of layer 1 (l1[0, m1), or all
 // its m1 hits when l1 is null), 128 of them at a time in registers: each hit k_first +
@@ -1360,6 +1490,31 @@ __device__ __forceinline__ void sieve_triples(const Job& j, W& w, uint32_t* pend
     }
 }
 
+// The same object and lane index, but not known to the compiler to be the same:
+// code that seldom runs then derives its addresses and masks for itself instead
+// of having them kept in registers for it all along.
+template <class V>
+__device__ __forceinline__ V& opaque_shared(V& v) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(&v);
+    asm volatile("" : "+r"(a));
+    return *reinterpret_cast<V*>(__cvta_shared_to_generic(a));
+}
+__device__ __forceinline__ int opaque_lane() {
+    int l;
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(l));
+    return l;
+}
+
+// Hits left of layer 2 beyond which a station is crowded: where the row lists cost
+// less than trying each of those hits with all of layer 1.  One warp, limits 8, 12
+// and 18: 20 000 events of 100 hits per layer with a 1 cm window 515, 526 and 555 us
+// (639 without row lists), 10^6 events with 0.5 cm, where few stations have as
+// many, 5.43, 5.33 and 5.33 ms.  A block shares those hits between four warps: 12, 16
+// and 24 differ by less than 3 %.  Row lists made events of 250 hits per layer with
+// a 1 cm window (medium path, 3 000 events) 357 us, 599 on the block tile and 818
+// without them; 200 hits 279, 554; 100 hits with 2 cm (warp path) 592, 1 401.
+constexpr int kCrowdedWarp = 12, kCrowdedBlock = 24;
+
 // Stages station s of event e and finds its triples (see above).  Returns 0, 1 for
 // a hit with z <= 0 or 2 for one whose pruning bound is not finite.
 template <bool EMIT>
@@ -1393,6 +1548,17 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
     static_assert(SmallCfg::LAYER_CAP <= 6 * 32, "rounds of a layer");
     m2 = uniform(m2);
     m0 = uniform(m0);
+    if (m2 > kCrowdedWarp) {
+        using Lists = RowLists<uint8_t, SmallCfg::LAYER_CAP, 1>;
+        static_assert(sizeof(Lists) <= sizeof(w.map), "the lists take the maps' memory");
+        WarpTile& v = opaque_shared(w);
+        const int ln = opaque_lane();
+        Lists& r = *reinterpret_cast<Lists*>(v.map);
+        row_lists<32>(r, v.P, ln, sb.inv, v.left[0], m0, (const uint8_t*)nullptr, n1, n0);
+        np = row_triples<EMIT>(j, v, v.pend, r, r.queue[0], ln, c, sb.B, sb.inv, e, s, n0, n0 + n1, v.left[1], m2, 0, 1,
+                               sink, np);
+        m2 = 0;
+    }
     if (m2 > 0 || (all && np > 0))
         sieve_triples<EMIT, false>(j, w, w.pend, lane, c, sb.B, e, s, n0, n0 + n1, w.left[0], m0,
                                    (const uint8_t*)nullptr, n1, w.left[1], m2, 0, 1, sink, all, np);
@@ -1964,9 +2130,8 @@ __device__ __forceinline__ void medium_pass(const Job& j, MediumTile& w, float i
 
 // Stages station s of the event in w.off and finds its triples (see
 // sieve_layers; a third map leaves fewer hits of layer 1 when layer 2 has more
-// than kFilterMin).  Returns 0, 1 for a hit with z <= 0, 2 for one whose pruning
-// bound is not finite or 3 for a station too dense for the sieve; block-uniform,
-// all threads call it.
+// than kFilterMin).  Returns 0, 1 for a hit with z <= 0 or 2 for one whose pruning
+// bound is not finite; block-uniform, all threads call it.
 constexpr int kFilterMin = 8;
 template <bool EMIT>
 __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const Cuts& c, int64_t e, int s, bool sink,
@@ -2041,7 +2206,6 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
         if (uniform(__syncthreads_or(wild))) return 2;
         reduce();
     }
-    if (!EMIT && uniform(too_dense(max(max(n0, n1), n2), sb.B))) return 3;
     for (int p0 = 0; p0 < n1; p0 += T) {
         const SieveBit b = medium_bit(w.P[s1 + p0 + tid], sb.inv);
         if (p0 + tid < n1) atomicOr(&ma[b.word], b.bit);
@@ -2061,7 +2225,16 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
         m1 = uniform(w.n_left[1]);
         l1 = w.left[1];
     }
-    sieve_triples<EMIT, true>(j, w, w.pend[wp], lane, c, sb.B, e, s, s1, s2, w.left[0], m0, l1, m1, w.left[2], m2, wp,
+    const bool crowded = m2 > kCrowdedBlock;
+    if (crowded) {
+        using Lists = RowLists<uint16_t, MediumCfg::LAYER_CAP, MediumTile::WARPS>;
+        static_assert(sizeof(Lists) <= sizeof(w.map), "the lists take the maps' memory");
+        Lists& r = *reinterpret_cast<Lists*>(w.map);
+        row_lists<T>(r, w.P, tid, sb.inv, w.left[0], m0, l1, m1, s1);
+        np = row_triples<EMIT>(j, w, w.pend[wp], r, r.queue[wp], lane, c, sb.B, sb.inv, e, s, s1, s2, w.left[2], m2, wp,
+                          MediumTile::WARPS, sink, np);
+    }
+    sieve_triples<EMIT, true>(j, w, w.pend[wp], lane, c, sb.B, e, s, s1, s2, w.left[0], m0, l1, m1, w.left[2], crowded ? 0 : m2, wp,
                               MediumTile::WARPS, sink, all, np);
     return 0;
 }
@@ -2102,7 +2275,7 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
                     atomicOr(&j.ctrl->status, kStInvalid);
                     j.ev_class[e] = kClsInvalid;
                 } else {
-                    push_event(j, e, st == 2 ? kClsGeneric : kClsHeavy);
+                    push_event(j, e, kClsGeneric);
                 }
             }
             return;

@@ -34,3 +34,104 @@ def test_offsets_whose_differences_wrap(lib, oracle_mod, mode, up, down):
         for form in ("plain", "batched"):
             assert gpu_select(ctx, b, form=form, triplets=False)["status"] == lib.JPSI_EINVAL, (at, form)
         ctx.close()
+
+
+def _oracle_same(lib, oracle_mod, b, S, t, modes=(0, 1), forms=("plain", "batched"), record_caps=(-1,), label=""):
+    from gpu_helpers import assert_same
+    for mode in modes:
+        ref = oracle_mod.run(oracle_mod.params(S, mode, t_xz=t, t_yz=t), b, n_threads=8)
+        assert ref["status"] == 0
+        ctx = lib.Context(lib.params(S, mode, t_xz=t, t_yz=t))
+        for cap in record_caps:
+            tu = lib.jpsi_get_tuning(ctx.ctx)
+            tu.record_cap = cap
+            assert lib.jpsi_set_tuning(ctx.ctx, tu) == lib.JPSI_OK
+            for form in forms:
+                assert_same(gpu_select(ctx, b, form=form), ref, b["n_events"] * S, label=f"{label} mode{mode} {form}")
+        ctx.close()
+
+
+def _clustered(rng, n, n_clusters, radius, spread, z):
+    """n hits of one layer in clusters of slopes (radius about their centres)."""
+    centres = rng.uniform(-spread, spread, (n_clusters, 2))
+    s = centres[rng.integers(n_clusters, size=n)] + rng.uniform(-radius, radius, (n, 2))
+    return list(zip(s[:, 0] * z, s[:, 1] * z, np.full(n, z)))
+
+
+# around the limits at which a station counts as crowded (12 hits on a warp, 24 on
+# a medium block), full rounds, and the largest layers of both paths
+@pytest.mark.parametrize("n", [12, 13, 24, 25, 33, 64, 100, 192, 200, 300, 384])
+def test_crowded_stations(lib, oracle_mod, n):
+    # clusters over more rows than a map has (they wrap around), over a few rows and
+    # over one; crowded trigger stations (PAPER) and crowded partners (CHAIN)
+    rng = np.random.default_rng(100 + n)
+    zl = layer_z(2)
+    events = []
+    for spread in (4.0, 0.3, 0.004):
+        for k in range(6):
+            clusters = max(1, n // 12)
+            # about one partner per hit: the clusters of a narrow spread are the spread
+            radius = 0.012 if spread > 0.01 else 0.02
+            seed = rng.integers(1 << 30)
+            ev = []
+            for s in range(2):
+                for l in range(3):
+                    full = (s == k % 2)
+                    r = np.random.default_rng(seed)  # the same clusters in every layer
+                    m = (n if n <= 128 or l == 1 else min(n, (384 if n <= 192 else 960) - n) // 2) if full else 4
+                    hits = _clustered(r, m, clusters, radius, spread, zl[3 * s + l])
+                    j = rng.uniform(-0.3, 0.3, (m, 2))
+                    ev.append([(x + dx, y + dy, z) for (x, y, z), (dx, dy) in zip(hits, j)])
+            events.append(ev)
+    b = make_batch(events, 2)
+    _oracle_same(lib, oracle_mod, b, 2, 0.04, record_caps=(-1, 0), label=f"n={n}")
+
+
+def _time_us(f, n=15):
+    import torch
+    best = float("inf")
+    for _ in range(n):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3)
+    return best
+
+
+def _selection(lib, b, S, mode, w):
+    """A call of the selection on the batch (numpy dict), window w cm, outputs on the device."""
+    import torch
+    d = {k: torch.from_numpy(np.ascontiguousarray(b[k])).cuda() for k in ("x", "y", "z", "offsets")}
+    ctx = lib.Context(lib.params(S, mode, t_xz=w * w, t_yz=w * w))
+    tracks = torch.zeros(b["n_events"], dtype=torch.int32, device="cuda")
+    o = lib.jpsi_outputs()
+    o.track_counts = tracks.data_ptr()
+    hb = lib.make_batch(d["x"], d["y"], d["z"], d["offsets"], b["n_events"])
+
+    def call():
+        call.keep = (ctx, d, tracks)
+        assert lib.jpsi_run(ctx.ctx, hb, o, torch.cuda.current_stream().cuda_stream) == 0
+    return call
+
+
+def _random_batch(n_events, S, n, seed, r_min=0.1, r_max=0.4):
+    """n hits per layer, radii log-uniform in slope, straight from the origin."""
+    rng = np.random.default_rng(seed)
+    z = np.tile(np.repeat(np.array(layer_z(S), np.float32), n), n_events)
+    r = r_min * (r_max / r_min) ** rng.random(len(z))
+    phi = rng.uniform(0, 2 * np.pi, len(z))
+    off = np.arange(n_events * 3 * S + 1, dtype=np.int32) * n
+    return {"x": (r * np.cos(phi) * z).astype(np.float32), "y": (r * np.sin(phi) * z).astype(np.float32), "z": z,
+            "offsets": off, "n_events": n_events, "n_hits": len(z), "n_stations": S}
+
+
+@pytest.mark.parametrize("S,n,narrow,wide,mode", [(1, 100, 0.5, 1.1, 0), (4, 200, 0.5, 1.0, 1), (4, 250, 0.5, 1.0, 1)])
+def test_wide_windows_keep_their_speed(lib, S, n, narrow, wide, mode):
+    # twice the window is 16 times the triplets but few of the work: 1.2 to 2.0
+    # times the time of the narrow one.  Hits tried each with each took 3 to 5.
+    b = _random_batch(6400000 // n // S, S, n, 5)
+    t = [_time_us(_selection(lib, b, S, mode, w)) for w in (narrow, wide)]
+    assert t[1] < 2.5 * t[0], t
