@@ -123,6 +123,9 @@ struct TileView {
 // 2, triples that wait for their fit, and the event's trigger slopes.
 constexpr int kMapRows = 128;             // a map has 128 rows (s_y) of 64 columns (s_x), both modulo
 constexpr int kMapWords = 2 * kMapRows;   // word 2 y + (x >> 5), bit x
+struct LayerMax {
+    float r, s;                           // largest 1/z and |slope| of a layer's live hits
+};
 struct WarpTile {
     static constexpr int TCAP = SmallCfg::TCAP;
     static constexpr uint8_t CLS = kClsLight;
@@ -139,6 +142,7 @@ struct WarpTile {
         float2 Tt[SmallCfg::TCAP];                // or their (min t, max t) (free-streaming windows)
     };
     uint8_t alive[SmallCfg::TCAP];
+    LayerMax lay[3];                      // of an uneven station
     static_assert(SmallCfg::LAYER_CAP <= 256, "8-bit indices");
 };
 
@@ -164,6 +168,7 @@ struct MediumTile {
         float2 Tt[TCAP];
     };
     uint8_t alive[TCAP];
+    LayerMax lay[3];                            // of an uneven station
     static_assert(MediumCfg::LAYER_CAP <= 512, "9-bit indices in pend");
 };
 
@@ -967,7 +972,7 @@ __device__ bool road_warp(const Job& j, const TV& t, const Cuts& c, float mx, fl
 
 // A warp-uniform value in a uniform register: branches and addresses that come
 // from it need no divergence handling (the compiler does not know that the
-// result of a shuffle is uniform; that of a reduction is).
+// result of a shuffle or of a load is uniform; that of a reduction is).
 __device__ __forceinline__ int uniform(int v) { return __reduce_max_sync(kFull, v); }
 
 // Largest |v| seen so far, NaN if any value was NaN.
@@ -995,40 +1000,74 @@ __device__ __forceinline__ StationBounds station_bounds(float rmax, float smax, 
     StationBounds sb;
     sb.B = station_pair_bound(rmax, smax, K);
     sb.b = __fadd_rn(__fadd_rn(__fmul_rn(K, rmax), __fmul_rn(2.0f * kKappa, smax)), kTau);
-    sb.inv = fminf(__fmul_rn(0.998f, rcp_approx(sb.B)), __fmul_rn(4096.0f, rcp_approx(smax)));
+    sb.inv = __fmul_rn(0.998f, rcp_approx(sb.B));
     return sb;
 }
 
-// Exact classification of the station's hits [o0, o0 + n), for stations with an
-// odd coordinate: their slopes to P, (Inf, Inf) for a hit with a non-finite
-// coordinate (it passes no finite bound, and no fit in any case).  Returns 0, 1
-// (z <= 0) or 2 (a hit whose pruning bound is not finite).
+// One bound serves a station whose hits are alike.  A single hit at a small z
+// or a huge slope would make it so wide that every triple of the station came to a
+// fit (one such hit in every other event of 100 hits per layer: 0.2 -> 45 ms); such
+// an uneven station gets a bound for each pair of its layers instead, as only the
+// two pairs with that hit's layer are then wide.  Alike: 1/z within a factor of
+// four, and slopes that add no more than a quarter to the bound (or below 8).
+__device__ __forceinline__ bool even_hits(int rmax_bits, int rmin_bits, float rmax, float smax, float K) {
+    return rmax_bits <= rmin_bits + (2 << 23) && smax <= fmaxf(8.0f, __fmul_rn(11585.0f * K, rmax));
+}
+
+// The bounds of the three pairs of layers.
+struct PairBounds {
+    float b01, b02, b12;
+};
+__device__ __forceinline__ bool uneven_bounds(const PairBounds& b, float B) {
+    return fminf(fminf(b.b01, b.b02), b.b12) < 0.5f * B;
+}
+__device__ __forceinline__ PairBounds pair_bounds(const LayerMax* lay, float K) {
+    const float b[3] = {lay[0].r, lay[1].r, lay[2].r}, m[3] = {lay[0].s, lay[1].s, lay[2].s};
+    return {station_pair_bound(fmaxf(b[0], b[1]), fmaxf(m[0], m[1]), K),
+            station_pair_bound(fmaxf(b[0], b[2]), fmaxf(m[0], m[2]), K),
+            station_pair_bound(fmaxf(b[1], b[2]), fmaxf(m[1], m[2]), K)};
+}
+
+// Exact classification of the station's hits (n places from o0 on), for stations
+// with an odd coordinate or uneven hits: their slopes to P, (Inf, Inf) for a hit
+// with a non-finite coordinate (it passes no finite bound, and no fit in any case),
+// and each layer's maxima to `lay`.  Returns 0, 1 (z <= 0) or 2 (a hit whose
+// pruning bound is not finite).
 __device__ __forceinline__ int sieve_classify(const Job& j, float2* P, int lane, int32_t o0, int s1, int s2, int n,
-                                              const Shift3& sh, float& rmax, float& smax) {
+                                              const Shift3& sh, LayerMax* lay, float& rmax, float& smax) {
     bool zbad = false, wild = false;
     rmax = smax = 0.0f;
     __syncwarp();  // (the slopes written so far)
 #pragma unroll 1
-    for (int p = lane; p < n; p += 32) {
-        const int32_t g = o0 + p + sh.at(p, s1, s2);
-        const HitPrep h = hit_prep(__ldg(j.x + g), __ldg(j.y + g), __ldg(j.z + g), j.K);
-        zbad |= h.zbad;
-        wild |= h.wild;
-        const bool live = h.live & !h.wild;
-        P[p] = live ? make_float2(h.sx, h.sy) : make_float2(INFINITY, INFINITY);
-        if (live) {
-            smax = fmaxf(smax, fmaxf(fabsf(h.sx), fabsf(h.sy)));
-            rmax = fmaxf(rmax, h.r);
+    for (int l = 0; l < 3; ++l) {
+        float r = 0.0f, sl = 0.0f;
+        const int end = l == 0 ? s1 : l == 1 ? s2 : n;
+#pragma unroll 1
+        for (int p = (l == 0 ? 0 : l == 1 ? s1 : s2) + lane; p < end; p += 32) {
+            const int32_t g = o0 + p + (kStream ? sh.of(l) : 0);
+            const HitPrep h = hit_prep(__ldg(j.x + g), __ldg(j.y + g), __ldg(j.z + g), j.K);
+            zbad |= h.zbad;
+            wild |= h.wild;
+            const bool live = h.live & !h.wild;
+            P[p] = live ? make_float2(h.sx, h.sy) : make_float2(INFINITY, INFINITY);
+            if (live) {
+                sl = fmaxf(sl, fmaxf(fabsf(h.sx), fabsf(h.sy)));
+                r = fmaxf(r, h.r);
+            }
         }
+        sl = __int_as_float(__reduce_max_sync(kFull, __float_as_int(sl)));
+        r = __int_as_float(__reduce_max_sync(kFull, __float_as_int(r)));
+        if (lane == 0) lay[l] = LayerMax{r, sl};
+        smax = fmaxf(smax, sl);
+        rmax = fmaxf(rmax, r);
     }
-    smax = __int_as_float(__reduce_max_sync(kFull, __float_as_int(smax)));
-    rmax = __int_as_float(__reduce_max_sync(kFull, __float_as_int(rmax)));
     __syncwarp();
     return __any_sync(kFull, zbad) ? 1 : __any_sync(kFull, wild) ? 2 : 0;
 }
 
 // The cell of a slope: the nearest integer of s * inv, modulo the map's size
-// when it is used.  |s * inv| <= 4096, so the sum with 1.5 * 2^23 holds that
+// when it is used.  A bound is at least 2 kappa times the largest |s| that it is
+// used on, so |s * inv| <= 2^16 (1 + 2^-20), and the sum with 1.5 * 2^23 holds that
 // integer in its low mantissa bits (one rounding).  Hits of one passing
 // triplet lie within B (1 - 5e-5) of each other (jpsi_device.cuh) and inv <=
 // 0.998 (1 + 2^-22) / B, so their s * inv differ by less than 1 and their
@@ -1153,7 +1192,7 @@ __device__ __forceinline__ int light_fit(const Job& j, W& w, const uint32_t* pen
 // turn, each of at most 32 R hits) to P, in the order of the hits, and the largest
 // 1/z and |slope|.  Returns false, P then incomplete, for hits that want
 // sieve_classify: NaN, an infinity or 1/z outside (2^-126, 2^126) among the hits
-// read, or a station so close to the end of the hit arrays that the lanes past
+// read, uneven hits (even_hits), or a station so close to the end of the hit arrays that the lanes past
 // the end of a layer, which read on into the hits behind it, would leave them.
 template <int R>
 __device__ __forceinline__ bool sieve_stage(const Job& j, WarpTile& w, int lane, int32_t o0, int n0, int n1, int n2,
@@ -1203,7 +1242,7 @@ __device__ __forceinline__ bool sieve_stage(const Job& j, WarpTile& w, int lane,
               ni = __reduce_min_sync(kFull, __float_as_int(rmin));
     smax = __int_as_float(si);
     rmax = __int_as_float(ri);
-    return si < 0x7f800000 && ri < 0x7e800000 && ni > 0x00800000;
+    return si < 0x7f800000 && ri < 0x7e800000 && ni > 0x00800000 && even_hits(ri, ni, rmax, smax, j.K);
 }
 
 // The sieve of the staged station: which hits of layers 0 and 2 can be part of a
@@ -1272,29 +1311,60 @@ __device__ __forceinline__ void sieve_layers(const Job& j, WarpTile& w, int lane
 }
 
 // Crowded stations (wide windows: the maps let most hits through).  Trying every
-// hit that is left with every other grows with the square of the hits, so there
-// layers 0 and 1 are put in the order of their cells' rows, and a hit looks at
-// three rows of them.  The lists take the maps' memory, which is free by then.
+// hit that is left with every other grows with the square of the hits, so there two
+// of the layers are put in the order of their cells' rows, and a hit looks at three
+// rows of them.  The hits of the outer layer find partners in the middle one (the
+// pair of layers with the tightest bound), those pairs find theirs in the last:
+// layers 2, 1 and 0 unless the hits are uneven.
 // Bound by instruction issue: two passes over the hits make the lists, then a step
 // of a walk is two loads, the pair test and a vote for 32 hits.
-//   L: the type of the indices; MAX: hits per layer; Q: pair queues (one per warp).
+//   The lists, and what a search keeps from one fit to the next, take the maps'
+// memory, which is free by then: in registers they cost the stations that never come
+// here 9 %.  Loops run to uniform() ends: one that the compiler cannot show to be
+// the same for all lanes makes it prepare every vote and reduction of the kernel for
+// diverged warps, which is half as much code again (k_light 58 -> 91 KB) and then a
+// wait for instructions (10^6 events 4.61 -> 5.5 to 6.4 ms).
+//   L: the type of the indices; MAX: hits per layer; Q: warps.
 constexpr int kRowQueue = 64;
+struct RowState {
+    // outer hits from `due` on have not looked, the next 32 of them from step t of
+    // their rows on; pairs waiting in the queue and, behind them, looking for
+    // partners, from step u of their rows on.  Kept as due | t << 10 | waiting << 20
+    // and looking | u << 8.
+    int due, t, waiting, looking, u;
+    __device__ __forceinline__ explicit RowState(const int2& p) {
+        const int a = uniform(p.x), b = uniform(p.y);
+        due = a & 1023;
+        t = a >> 10 & 1023;
+        waiting = a >> 20;
+        looking = b & 255;
+        u = b >> 8;
+    }
+    __device__ __forceinline__ int2 packed() const {
+        return make_int2(due | t << 10 | waiting << 20, looking | u << 8);
+    }
+};
 template <class L, int MAX, int Q>
 struct RowLists {
-    uint32_t end[2][kMapRows];  // where each row's hits end (layer 0, layer 1)
-    L order[2][MAX];            // layer-local indices by row
-    uint32_t queue[Q][kRowQueue];  // pairs: j << 9 | k
+    uint32_t end[2][kMapRows];     // where each row's hits end (middle, last layer)
+    L order[2][MAX];               // layer-local indices by row
+    uint32_t queue[Q][kRowQueue];  // pairs, as they stand in the pending triples
+    int2 state[Q];                 // RowState, packed
+    int n_out, start[3], shift[3];  // hits of the outer layer; places and index shifts of outer, middle and last
+    float b, b_out, b_mid;          // bounds of the pairs outer - middle, outer - last, middle - last
+    float inv[2];                   // cells per unit of slope of middle and last
+    bool from_out;                  // partners in the last layer are looked for around the outer hit
 };
 
 // The row of a hit's cell.
 __device__ __forceinline__ int sieve_row(float2 s, float inv) { return sieve_cell(s.y, inv) & (kMapRows - 1); }
 
-// Fills the lists from m0 hits of layer 0 (l0) and m1 of layer 1 (l1, or all of
-// them when it is null), whose slopes start at places 0 and s1.  All T threads
-// (a warp or a block) call it.
+// Fills the lists from m0, m1, m2 hits of the layers, whose indices are in `left` from
+// 0, f1 and f2 on (all of layer 1 when f1 < 0) and whose slopes start at places 0, s1
+// and s2.  All T threads (a warp or a block) call it.
 template <int T, class R, class L>
-__device__ __forceinline__ void row_lists(R& r, const float2* P, int tid, float inv, const L* l0, int m0, const L* l1,
-                                          int m1, int s1) {
+__device__ __forceinline__ void row_lists(const Job& j, R& r, const float2* P, int tid, const PairBounds& pb,
+                                          const L* left, int m0, int f1, int m1, int f2, int m2, int s1, int s2) {
     auto sync = [] {
         if constexpr (T == 32)
             __syncwarp();
@@ -1302,34 +1372,60 @@ __device__ __forceinline__ void row_lists(R& r, const float2* P, int tid, float 
             __syncthreads();
     };
     const int lane = tid & 31;
+    const bool from0 = pb.b01 < pb.b12 && pb.b01 <= pb.b02, over1 = pb.b02 < pb.b12 && pb.b02 < pb.b01;
+    const int f_mid = over1 ? 0 : f1, f_last = over1 ? f1 : from0 ? f2 : 0;
+    const int n_mid = over1 ? m0 : m1, n_last = over1 ? m1 : from0 ? m2 : m0;
+    const int p_mid = over1 ? 0 : s1, p_last = over1 ? s1 : from0 ? s2 : 0;
     sync();  // the maps are done with
     for (int q = tid; q < 2 * kMapRows; q += T) r.end[0][q] = 0u;
-    sync();
-#pragma unroll 1
-    for (int q = tid; q < m0 + m1; q += T) {
-        const bool a = q < m0;
-        const int h = a ? l0[q] : l1 ? l1[q - m0] : q - m0;
-        atomicAdd(&r.end[a ? 0 : 1][sieve_row(P[a ? h : s1 + h], inv)], 1u);
+    if (tid < T / 32) r.state[tid] = make_int2(tid, 0);
+    if (tid == 0) {
+        r.n_out = from0 ? m0 : m2;
+        const int out_l = from0 ? 0 : 2, mid_l = over1 ? 0 : 1, last_l = 3 - out_l - mid_l;
+        r.start[0] = from0 ? 0 : s2;
+        r.start[1] = p_mid;
+        r.start[2] = p_last;
+        r.shift[0] = 18 - 9 * out_l;
+        r.shift[1] = 18 - 9 * mid_l;
+        r.shift[2] = 18 - 9 * last_l;
+        r.b = over1 ? pb.b02 : from0 ? pb.b01 : pb.b12;
+        r.b_out = over1 ? pb.b12 : pb.b02;
+        r.b_mid = over1 || !from0 ? pb.b01 : pb.b12;
+        r.from_out = r.b_out < r.b_mid;
+        r.inv[0] = __fmul_rn(0.998f, rcp_approx(r.b));
+        r.inv[1] = __fmul_rn(0.998f, rcp_approx(fminf(r.b_out, r.b_mid)));
     }
     sync();
-    // rows' starts (four rows a lane); placing the hits turns them into ends
-    if (tid < 32) {
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-            uint4* p = reinterpret_cast<uint4*>(r.end[l]) + lane;
-            const uint4 c = *p;
-            const uint32_t b = (uint32_t)warp_incl_scan((int)(c.x + c.y + c.z + c.w), lane) - (c.x + c.y + c.z + c.w);
-            *p = make_uint4(b, b + c.x, b + c.x + c.y, b + c.x + c.y + c.z);
+    // twice over the hits: each row's size, then their places (which turn the rows'
+    // starts into their ends)
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+        for (int w = 0; w < 2; ++w) {
+            const int f = w ? f_last : f_mid, n = uniform(w ? n_last : n_mid);
+            const float2* slopes = P + (w ? p_last : p_mid);
+            const float inv = r.inv[w];
+#pragma unroll 1
+            for (int q0 = 0; q0 < n; q0 += T) {
+                const int q = q0 + tid;
+                if (q >= n) continue;
+                const int h = f >= 0 ? (int)left[f + q] : q;
+                const uint32_t at = atomicAdd(&r.end[w][sieve_row(slopes[h], inv)], 1u);
+                if (pass && JPSI_IN(j.ctrl, at < sizeof(r.order[0]) / sizeof(L))) r.order[w][at] = (L)h;
+            }
         }
+        sync();
+        if (!pass && (T == 32 || tid < 32)) {  // four rows a lane
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                uint4* p = reinterpret_cast<uint4*>(r.end[w]) + lane;
+                const uint4 c = *p;
+                const uint32_t sum = c.x + c.y + c.z + c.w, b = (uint32_t)warp_incl_scan((int)sum, lane) - sum;
+                *p = make_uint4(b, b + c.x, b + c.x + c.y, b + c.x + c.y + c.z);
+            }
+        }
+        if (!pass) sync();
     }
-    sync();
-#pragma unroll 1
-    for (int q = tid; q < m0 + m1; q += T) {
-        const bool a = q < m0;
-        const int h = a ? l0[q] : l1 ? l1[q - m0] : q - m0;
-        r.order[a ? 0 : 1][atomicAdd(&r.end[a ? 0 : 1][sieve_row(P[a ? h : s1 + h], inv)], 1u)] = (L)h;
-    }
-    sync();
 }
 
 // The hits of a row and of the rows beside it (a ring): up to two runs of the order.
@@ -1347,69 +1443,84 @@ __device__ __forceinline__ RowRuns row_runs(const uint32_t* end, int row) {
     return w;
 }
 
-// The triples of a crowded station (see sieve_triples, whose pending triples and
-// fits they share): 32 hits of l2 at a time (k_first + k_step (32 b + lane)) look
-// for partners in their rows of layer 1, and 32 of the pairs found for partners in
-// theirs of layer 0, each lane walking its own runs.
-template <bool EMIT, class W, class R, class L>
-__device__ __forceinline__ int row_triples(const Job& j, W& w, uint32_t* pend, const R& r, uint32_t* queue, int lane,
-                                            const Cuts& c, float B, float inv, int64_t e, int s, int s1, int s2,
-                                            const L* l2, int m2, int k_first, int k_step, bool sink, int np) {
+// Searches on until more than 32 triples (np) are pending or, then returning false,
+// to the end: 32 hits of the outer layer at a time (this warp's are wp + k_step (32 b +
+// lane)) look for partners in their rows, and 32 of the pairs found for theirs, each
+// lane walking its own runs.
+template <class R, class L>
+__device__ __forceinline__ bool row_search(const Job& j, const float2* P, uint32_t* pend, R& r, int wp, int k_step,
+                                           uint32_t station, const L* l0, const L* l2, int lane, int& np) {
     const uint32_t lt = (1u << lane) - 1u;
-    // what lives on across a fit: the hits of l2 from kb on are due, from step t of
-    // their runs; qn pairs wait; behind them dn are looking for partners, from step u
-    int kb = k_first, t = 0, qn = 0, dn = 0, u = 0;
+    uint32_t* queue = r.queue[wp];
+    RowState st(r.state[wp]);
+    const int so = r.shift[0], sm = r.shift[1], sl = r.shift[2];
+    const float2 *outer = P + r.start[0], *middle = P + r.start[1], *last = P + r.start[2];
+    bool more = true;
 #pragma unroll 1
-    for (;;) {
-        if (dn == 0) {
+    do {
+        if (st.looking == 0) {
+            const int n = uniform(r.n_out);
+            const L* out = so ? l0 : l2;
 #pragma unroll 1
-            while (qn < 32 && kb < m2) {
-                const int k = kb + k_step * lane;
-                const int hk = l2[min(k, m2 - 1)];
-                const float2 Pk = w.P[s2 + hk];
-                const RowRuns rk = row_runs(r.end[1], sieve_row(Pk, inv));
-                const int len = k < m2 ? rk.len : 0, steps = __reduce_max_sync(kFull, len);
+            while (st.waiting < 32 && st.due < n) {
+                const int k = st.due + k_step * lane;
+                const int ho = out[min(k, n - 1)];
+                const float2 O = outer[ho];
+                const RowRuns w = row_runs(r.end[0], sieve_row(O, r.inv[0]));
+                const int len = k < n ? w.len : 0, steps = __reduce_max_sync(kFull, len);
+                const float B = r.b;
 #pragma unroll 1
-                for (; t < steps && qn < 32; ++t) {
-                    const bool in = t < len;
-                    const int hj = r.order[1][in ? rk.at(t) : 0];
-                    const float2 Pj = w.P[s1 + hj];
-                    const bool pass = in & pair_ok(Pj.x, Pj.y, Pk.x, Pk.y, B);
+                for (; st.t < steps && st.waiting < 32; ++st.t) {
+                    const bool in = st.t < len;
+                    const int hm = r.order[0][in ? w.at(st.t) : 0];
+                    const float2 M = middle[hm];
+                    const bool pass = in & pair_ok(M.x, M.y, O.x, O.y, B);
                     const unsigned mask = __ballot_sync(kFull, pass);
-                    const int at = qn + __popc(mask & lt);
-                    if (pass && JPSI_IN(j.ctrl, at < kRowQueue)) queue[at] = (uint32_t)hj << 9 | (uint32_t)hk;
-                    qn += __popc(mask);
+                    const int at = st.waiting + __popc(mask & lt);
+                    if (pass && JPSI_IN(j.ctrl, at < kRowQueue)) queue[at] = (uint32_t)ho << so | (uint32_t)hm << sm;
+                    st.waiting += __popc(mask);
                 }
-                if (t >= steps) {
-                    kb += 32 * k_step;
-                    t = 0;
+                const int both = uniform(st.waiting | st.t << 8);
+                st.waiting = both & 255;
+                st.t = both >> 8;
+                if (st.t >= steps) {
+                    st.due += 32 * k_step;
+                    st.t = 0;
                 }
             }
-            if (qn == 0) break;
-            dn = min(qn, 32);
-            qn -= dn;
-            u = 0;
+            if (st.waiting == 0) {
+                more = false;
+                break;
+            }
+            st.looking = min(st.waiting, 32);
+            st.waiting -= st.looking;
+            st.u = 0;
             __syncwarp();
         }
-        const uint32_t en = queue[qn + min(lane, dn - 1)];
-        const float2 Qj = w.P[s1 + (int)(en >> 9)], Qk = w.P[s2 + (int)(en & 511u)];
-        const RowRuns ri = row_runs(r.end[0], sieve_row(Qj, inv));
-        const int len = lane < dn ? ri.len : 0, steps = __reduce_max_sync(kFull, len);
+        const uint32_t en = queue[st.waiting + min(lane, st.looking - 1)];
+        const float2 O = outer[en >> so & 511u], M = middle[en >> sm & 511u];
+        const RowRuns w = row_runs(r.end[1], sieve_row(r.from_out ? O : M, r.inv[1]));
+        const int len = lane < st.looking ? w.len : 0, steps = __reduce_max_sync(kFull, len);
+        const float bo = r.b_out, bm = r.b_mid;
 #pragma unroll 1
-        for (; u < steps && np <= 32; ++u) {
-            const bool in = u < len;
-            const int hi = r.order[0][in ? ri.at(u) : 0];
-            const float2 Pi = w.P[hi];
-            const bool cand = in & pair_ok(Pi.x, Pi.y, Qj.x, Qj.y, B) & pair_ok(Pi.x, Pi.y, Qk.x, Qk.y, B);
+        for (; st.u < steps && np <= 32; ++st.u) {
+            const bool in = st.u < len;
+            const int hl = r.order[1][in ? w.at(st.u) : 0];
+            const float2 Z = last[hl];
+            const bool cand = in & pair_ok(Z.x, Z.y, O.x, O.y, bo) & pair_ok(Z.x, Z.y, M.x, M.y, bm);
             const unsigned mask = __ballot_sync(kFull, cand);
             const int at = np + __popc(mask & lt);
-            if (cand && JPSI_IN(j.ctrl, at < 64)) pend[at] = (uint32_t)s << 27 | (uint32_t)hi << 18 | en;
+            if (cand && JPSI_IN(j.ctrl, at < 64)) pend[at] = station | en | (uint32_t)hl << sl;
             np += __popc(mask);
         }
-        if (u >= steps) dn = 0;
-        np = light_fit<EMIT>(j, w, pend, lane, c, e, sink, uniform(np), 32);
-    }
-    return uniform(np);
+        const int both = uniform(np | st.u << 8);
+        np = both & 255;
+        st.u = both >> 8;
+        if (st.u >= steps) st.looking = 0;
+    } while (np <= 32);
+    __syncwarp();
+    if (lane == 0) r.state[wp] = st.packed();
+    return more;
 }
 
 // The triples whose pairs are all close enough, among the hits that the sieve
@@ -1418,12 +1529,12 @@ __device__ __forceinline__ int row_triples(const Job& j, W& w, uint32_t* pend, c
 // i k_step of l2 against layer 1, each pair found against l0.  They join the warp's
 // pending triples (np), which are fitted 32 at a time, or at the end of the station
 // when `all` is set: the fits of an event's non-trigger stations share their
-// instructions.
-template <bool EMIT, bool FILTER, class W, class L>
+// instructions.  A crowded station's are found from its row lists instead.
+template <bool EMIT, bool FILTER, class W, class R, class L>
 __device__ __forceinline__ void sieve_triples(const Job& j, W& w, uint32_t* pend, int lane, const Cuts& c, float B,
                                               int64_t e, int s, int s1, int s2, const L* l0, int m0, const L* l1,
                                               int m1, const L* l2, int m2, int k_first, int k_step, bool sink,
-                                              bool all, int& np) {
+                                              bool all, bool crowded, R& rows, int& np) {
     const uint32_t lt = (1u << lane) - 1u;
     const int hi0 = l0[min(lane, max(m0 - 1, 0))];  // what is left of layer 0, its first 32
     const float2 Pi0 = w.P[m0 > 0 ? hi0 : 0];
@@ -1432,77 +1543,66 @@ __device__ __forceinline__ void sieve_triples(const Job& j, W& w, uint32_t* pend
     unsigned mine = 0;                               // this lane's rounds with further partners of hk
     bool more = m2 > k_first;
     for (;;) {
+        if (__builtin_expect(crowded, 0)) {
+            more = uniform(row_search(j, w.P, pend, rows, k_first, k_step, (uint32_t)s << 27, l0, l2, lane, np));
+        } else {
 #pragma unroll 1
-        while (more && np <= 32) {
-            if (i0 >= m0) {
-                const unsigned lanes = __ballot_sync(kFull, mine != 0);
-                if (lanes) {  // the next pair
-                    const int from = __ffs(lanes) - 1;
-                    hj = j0 + 32 * (__ffs(__shfl_sync(kFull, mine, from)) - 1) + from;
-                    if (lane == from) mine &= mine - 1;
-                    if (hj < m1) {  // (an infinite bound lets the places past the end through)
-                        if (FILTER && l1) hj = l1[hj];
-                        Q = w.P[s1 + hj];
-                        i0 = 0;
-                    }
-                } else {
-                    k += k_step;
-                    if (k >= m2) {  // the next 128 hits of layer 1
-                        j0 += 128;
-                        if (j0 >= m1) {
-                            more = false;
-                            continue;
+            while (more && np <= 32) {
+                if (i0 >= m0) {
+                    const unsigned lanes = __ballot_sync(kFull, mine != 0);
+                    if (lanes) {  // the next pair
+                        const int from = __ffs(lanes) - 1;
+                        hj = j0 + 32 * (__ffs(__shfl_sync(kFull, mine, from)) - 1) + from;
+                        if (lane == from) mine &= mine - 1;
+                        if (hj < m1) {  // (an infinite bound lets the places past the end through)
+                            if (FILTER && l1) hj = l1[hj];
+                            Q = w.P[s1 + hj];
+                            i0 = 0;
                         }
-                        k = k_first;
+                    } else {
+                        k += k_step;
+                        if (k >= m2) {  // the next 128 hits of layer 1
+                            j0 += 128;
+                            if (j0 >= m1) {
+                                more = false;
+                                continue;
+                            }
+                            k = k_first;
 #pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            const int p = j0 + 32 * r + lane;
-                            const int h = min(p, m1 - 1);
-                            Pj[r] = w.P[s1 + (FILTER && l1 ? (int)l1[h] : h)];
-                            if (p >= m1) Pj[r].x = INFINITY;
+                            for (int r = 0; r < 4; ++r) {
+                                const int p = j0 + 32 * r + lane;
+                                const int h = min(p, m1 - 1);
+                                Pj[r] = w.P[s1 + (FILTER && l1 ? (int)l1[h] : h)];
+                                if (p >= m1) Pj[r].x = INFINITY;
+                            }
                         }
-                    }
-                    hk = l2[k];
-                    Pk = w.P[s2 + hk];
+                        hk = l2[k];
+                        Pk = w.P[s2 + hk];
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) mine |= pair_ok(Pj[r].x, Pj[r].y, Pk.x, Pk.y, B) ? 1u << r : 0u;
+                        for (int r = 0; r < 4; ++r) mine |= pair_ok(Pj[r].x, Pj[r].y, Pk.x, Pk.y, B) ? 1u << r : 0u;
+                    }
+                    continue;
                 }
-                continue;
+                int hi = hi0;
+                float2 Pi = Pi0;
+                if (i0 > 0) {
+                    hi = l0[min(i0 + lane, m0 - 1)];
+                    Pi = w.P[hi];
+                }
+                const bool cand =
+                    (i0 + lane < m0) & pair_ok(Pi.x, Pi.y, Q.x, Q.y, B) & pair_ok(Pi.x, Pi.y, Pk.x, Pk.y, B);
+                const unsigned mask = __ballot_sync(kFull, cand);
+                const int at = np + __popc(mask & lt);
+                if (cand && JPSI_IN(j.ctrl, at < 64))
+                    pend[at] = (uint32_t)s << 27 | (uint32_t)hi << 18 | (uint32_t)hj << 9 | (uint32_t)hk;
+                np += __popc(mask);
+                i0 += 32;
             }
-            int hi = hi0;
-            float2 Pi = Pi0;
-            if (i0 > 0) {
-                hi = l0[min(i0 + lane, m0 - 1)];
-                Pi = w.P[hi];
-            }
-            const bool cand =
-                (i0 + lane < m0) & pair_ok(Pi.x, Pi.y, Q.x, Q.y, B) & pair_ok(Pi.x, Pi.y, Pk.x, Pk.y, B);
-            const unsigned mask = __ballot_sync(kFull, cand);
-            const int at = np + __popc(mask & lt);
-            if (cand && JPSI_IN(j.ctrl, at < 64))
-                pend[at] = (uint32_t)s << 27 | (uint32_t)hi << 18 | (uint32_t)hj << 9 | (uint32_t)hk;
-            np += __popc(mask);
-            i0 += 32;
         }
         np = uniform(np);
         np = light_fit<EMIT>(j, w, pend, lane, c, e, sink, np, all && !more ? 0 : 32);
         if (!more) break;
     }
-}
-
-// The same object and lane index, but not known to the compiler to be the same:
-// code that seldom runs then derives its addresses and masks for itself instead
-// of having them kept in registers for it all along.
-template <class V>
-__device__ __forceinline__ V& opaque_shared(V& v) {
-    uint32_t a = (uint32_t)__cvta_generic_to_shared(&v);
-    asm volatile("" : "+r"(a));
-    return *reinterpret_cast<V*>(__cvta_shared_to_generic(a));
-}
-__device__ __forceinline__ int opaque_lane() {
-    int l;
-    asm volatile("mov.u32 %0, %%laneid;" : "=r"(l));
-    return l;
 }
 
 // Hits left of layer 2 beyond which a station is crowded: where the row lists cost
@@ -1511,8 +1611,8 @@ __device__ __forceinline__ int opaque_lane() {
 // (639 without row lists), 10^6 events with 0.5 cm, where few stations have as
 // many, 5.43, 5.33 and 5.33 ms.  A block shares those hits between four warps: 12, 16
 // and 24 differ by less than 3 %.  Row lists made events of 250 hits per layer with
-// a 1 cm window (medium path, 3 000 events) 357 us, 599 on the block tile and 818
-// without them; 200 hits 279, 554; 100 hits with 2 cm (warp path) 592, 1 401.
+// a 1 cm window (medium path, 3 000 events) 376 us, 599 on the block tile and 818
+// without them; 200 hits 297, 554; 100 hits with 2 cm (warp path) 592, 1 401.
 constexpr int kCrowdedWarp = 12, kCrowdedBlock = 24;
 
 // Stages station s of event e and finds its triples (see above).  Returns 0, 1 for
@@ -1525,7 +1625,7 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
     const Shift3 sh = kStream ? Shift3{uniform(w.sh[3 * s]), uniform(w.sh[3 * s + 1]), uniform(w.sh[3 * s + 2])}
                               : Shift3{0, 0, 0};
     float rmax, smax;
-    bool ok;
+    bool ok, uneven = false;
     if (most <= 64)
         ok = sieve_stage<2>(j, w, lane, o0, n0, n1, n2, sh, rmax, smax);
     else if (most <= 128)
@@ -1533,10 +1633,11 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
     else
         ok = sieve_stage<6>(j, w, lane, o0, n0, n1, n2, sh, rmax, smax);
     sb = station_bounds(rmax, smax, j.K);
-    if (!uniform(ok && sb.B < INFINITY)) {
-        const int st = uniform(sieve_classify(j, w.P, lane, o0, n0, n0 + n1, n0 + n1 + n2, sh, rmax, smax));
+    if (__builtin_expect(!uniform(ok && sb.B < INFINITY), 0)) {
+        const int st = uniform(sieve_classify(j, w.P, lane, o0, n0, n0 + n1, n0 + n1 + n2, sh, w.lay, rmax, smax));
         if (st) return st;
         sb = station_bounds(rmax, smax, j.K);
+        uneven = uniform(uneven_bounds(pair_bounds(w.lay, j.K), sb.B));
     }
     int m0, m2;
     if (most <= 64)
@@ -1548,20 +1649,16 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
     static_assert(SmallCfg::LAYER_CAP <= 6 * 32, "rounds of a layer");
     m2 = uniform(m2);
     m0 = uniform(m0);
-    if (m2 > kCrowdedWarp) {
-        using Lists = RowLists<uint8_t, SmallCfg::LAYER_CAP, 1>;
-        static_assert(sizeof(Lists) <= sizeof(w.map), "the lists take the maps' memory");
-        WarpTile& v = opaque_shared(w);
-        const int ln = opaque_lane();
-        Lists& r = *reinterpret_cast<Lists*>(v.map);
-        row_lists<32>(r, v.P, ln, sb.inv, v.left[0], m0, (const uint8_t*)nullptr, n1, n0);
-        np = row_triples<EMIT>(j, v, v.pend, r, r.queue[0], ln, c, sb.B, sb.inv, e, s, n0, n0 + n1, v.left[1], m2, 0, 1,
-                               sink, np);
-        m2 = 0;
-    }
+    using Lists = RowLists<uint8_t, SmallCfg::LAYER_CAP, 1>;
+    static_assert(sizeof(Lists) <= sizeof(w.map), "the lists take the maps' memory");
+    Lists& rows = *reinterpret_cast<Lists*>(w.map);
+    const bool crowded = uniform(m2 > (uneven ? 0 : kCrowdedWarp));
+    if (__builtin_expect(crowded, 0))
+        row_lists<32>(j, rows, w.P, lane, uneven ? pair_bounds(w.lay, j.K) : PairBounds{sb.B, sb.B, sb.B}, w.left[0],
+                      m0, -1, n1, SmallCfg::LAYER_CAP, m2, n0, n0 + n1);
     if (m2 > 0 || (all && np > 0))
         sieve_triples<EMIT, false>(j, w, w.pend, lane, c, sb.B, e, s, n0, n0 + n1, w.left[0], m0,
-                                   (const uint8_t*)nullptr, n1, w.left[1], m2, 0, 1, sink, all, np);
+                                   (const uint8_t*)nullptr, n1, w.left[1], m2, 0, 1, sink, all, crowded, rows, np);
     return 0;
 }
 
@@ -1581,7 +1678,7 @@ __device__ bool sieve_road(const Job& j, const W& w, int lane, const Cuts& c, co
             const int32_t h = g + p0 + lane;
             in = tube_pass(__ldg(j.x + h), __ldg(j.y + h), __ldg(j.z + h), mx, my, c);
         }
-        return __ballot_sync(kFull, in);
+        return (unsigned)uniform((int)__ballot_sync(kFull, in));
     };
 #pragma unroll 1
     for (int i0 = 0; i0 < n0; i0 += 32) {
@@ -1610,7 +1707,7 @@ __device__ bool sieve_road(const Job& j, const W& w, int lane, const Cuts& c, co
                                 ok = ok && partner_coincident(pmin, pmax, Tt, j.dt);
                             }
                         }
-                        if (__any_sync(kFull, ok)) return true;
+                        if (uniform(__any_sync(kFull, ok))) return true;
                     }
                 }
             }
@@ -1726,7 +1823,7 @@ __device__ void light_event_count(const Job& j, WarpTile& w, int lane, const Cut
             } else {
 #pragma unroll 1
                 for (int ti = 0; ti < nT; ++ti) {  // (CHAIN only: PAPER has one station)
-                    if (!w.alive[ti]) continue;
+                    if (!uniform(w.alive[ti])) continue;  // (uniform: see RowLists)
                     const float2 m = w.T[ti];
                     const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, shift3(w.sh, s), m.x, m.y,
                                                   kStream ? w.Tt[ti] : make_float2(0.f, 0.f));
@@ -1796,14 +1893,14 @@ __device__ __forceinline__ void light_event(const Job& j, WarpTile& w, int lane,
 
 // The warp path: every event of the batch (statically one warp per event, or
 // persistent warps grabbing `grab` events at a time).
-//   Bound by instruction issue (0.72 of the slots, ALU pipe the busiest) and, in
-// the loads of a station, by memory: 4 460 warp instructions per event of the
+//   Bound by instruction issue (0.70 of the slots, ALU pipe the busiest) and, in
+// the loads of a station, by memory: 4 370 warp instructions per event of the
 // 10^6-event workload, where sorting every hit into cells and walking windows of
-// them took 10 200.  10^6 events: 10.41 -> 4.73 ms (3.06 TB/s of hits, 0.46 of
+// them took 10 200.  10^6 events: 10.41 -> 4.61 ms (3.14 TB/s of hits, 0.47 of
 // the measured copy rate); the events of a 55 000-event log-normal timeslice that
-// fit: 0.394 -> 0.209 ms; 80 000 events in PAPER mode: 0.212 -> 0.108 ms.
-//   72 registers (28 warps per SM): 4.73 ms, against 4.86 with 64 (32 warps, a
-// few spills) and 80 (24 warps) and 5.40 with 56.
+// fit: 0.394 -> 0.208 ms; 80 000 events in PAPER mode: 0.212 -> 0.105 ms.
+//   72 registers (28 warps per SM) were measured before the row lists: 4.73 ms,
+// against 4.86 with 64 (32 warps, a few spills) and 80 (24 warps) and 5.40 with 56.
 template <bool EMIT>
 __global__ void __maxnreg__(72) k_light(const __grid_constant__ Job j) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2181,30 +2278,49 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
         smax = __int_as_float(bs);
         rmax = __int_as_float(br);
         sb = station_bounds(rmax, smax, j.K);
-        return bs < 0x7f800000 && br < 0x7e800000 && bn > 0x00800000 && sb.B < INFINITY;
+        return bs < 0x7f800000 && br < 0x7e800000 && bn > 0x00800000 && sb.B < INFINITY &&
+               even_hits(br, bn, rmax, smax, j.K);
     };
     uint32_t *ma = w.map[0], *mb = w.map[1];
 #pragma unroll
     for (int q = 0; q < 2 * kMapRows / T; ++q) reinterpret_cast<uint4*>(w.map)[T * q + tid] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < 3) w.n_left[tid] = 0;
-    if (!uniform(reduce())) {  // some odd coordinate: classify every hit exactly (see sieve_classify)
+    bool uneven = false;
+    if (!uniform(reduce())) {  // odd coordinates or uneven hits: classify every hit exactly (see sieve_classify)
         bool zbad = false, wild = false;
         smax = rmax = 0.0f;
-        for (int p = tid; p < n; p += T) {
-            const int32_t g = o0 + p + sh.at(p, s1, s2);
-            const HitPrep h = hit_prep(__ldg(j.x + g), __ldg(j.y + g), __ldg(j.z + g), j.K);
-            zbad |= h.zbad;
-            wild |= h.wild;
-            const bool live = h.live & !h.wild;
-            w.P[p] = live ? make_float2(h.sx, h.sy) : make_float2(INFINITY, INFINITY);
-            if (live) {
-                smax = fmaxf(smax, fmaxf(fabsf(h.sx), fabsf(h.sy)));
-                rmax = fmaxf(rmax, h.r);
+        if (tid < 3) w.lay[tid] = LayerMax{0.0f, 0.0f};
+        __syncthreads();
+#pragma unroll 1
+        for (int l = 0; l < 3; ++l) {
+            float r = 0.0f, sl = 0.0f;
+            const int end = l == 0 ? s1 : l == 1 ? s2 : n;
+#pragma unroll 1
+            for (int p = (l == 0 ? 0 : l == 1 ? s1 : s2) + tid; p < end; p += T) {
+                const int32_t g = o0 + p + (kStream ? sh.of(l) : 0);
+                const HitPrep h = hit_prep(__ldg(j.x + g), __ldg(j.y + g), __ldg(j.z + g), j.K);
+                zbad |= h.zbad;
+                wild |= h.wild;
+                const bool live = h.live & !h.wild;
+                w.P[p] = live ? make_float2(h.sx, h.sy) : make_float2(INFINITY, INFINITY);
+                if (live) {
+                    sl = fmaxf(sl, fmaxf(fabsf(h.sx), fabsf(h.sy)));
+                    r = fmaxf(r, h.r);
+                }
+            }
+            smax = fmaxf(smax, sl);
+            rmax = fmaxf(rmax, r);
+            // (values >= 0 order like their bit patterns)
+            const int ri = __reduce_max_sync(kFull, __float_as_int(r)), si = __reduce_max_sync(kFull, __float_as_int(sl));
+            if (lane == 0) {
+                atomicMax(reinterpret_cast<int*>(&w.lay[l].r), ri);
+                atomicMax(reinterpret_cast<int*>(&w.lay[l].s), si);
             }
         }
         if (uniform(__syncthreads_or(zbad))) return 1;
         if (uniform(__syncthreads_or(wild))) return 2;
         reduce();
+        uneven = uniform(uneven_bounds(pair_bounds(w.lay, j.K), sb.B));
     }
     for (int p0 = 0; p0 < n1; p0 += T) {
         const SieveBit b = medium_bit(w.P[s1 + p0 + tid], sb.inv);
@@ -2225,17 +2341,15 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
         m1 = uniform(w.n_left[1]);
         l1 = w.left[1];
     }
-    const bool crowded = m2 > kCrowdedBlock;
-    if (crowded) {
-        using Lists = RowLists<uint16_t, MediumCfg::LAYER_CAP, MediumTile::WARPS>;
-        static_assert(sizeof(Lists) <= sizeof(w.map), "the lists take the maps' memory");
-        Lists& r = *reinterpret_cast<Lists*>(w.map);
-        row_lists<T>(r, w.P, tid, sb.inv, w.left[0], m0, l1, m1, s1);
-        np = row_triples<EMIT>(j, w, w.pend[wp], r, r.queue[wp], lane, c, sb.B, sb.inv, e, s, s1, s2, w.left[2], m2, wp,
-                          MediumTile::WARPS, sink, np);
-    }
-    sieve_triples<EMIT, true>(j, w, w.pend[wp], lane, c, sb.B, e, s, s1, s2, w.left[0], m0, l1, m1, w.left[2], crowded ? 0 : m2, wp,
-                              MediumTile::WARPS, sink, all, np);
+    using Lists = RowLists<uint16_t, MediumCfg::LAYER_CAP, MediumTile::WARPS>;
+    static_assert(sizeof(Lists) <= sizeof(w.map), "the lists take the maps' memory");
+    Lists& rows = *reinterpret_cast<Lists*>(w.map);
+    const bool crowded = m2 > (uneven ? 0 : kCrowdedBlock);
+    if (crowded)
+        row_lists<T>(j, rows, w.P, tid, uneven ? pair_bounds(w.lay, j.K) : PairBounds{sb.B, sb.B, sb.B}, w.left[0], m0,
+                     l1 ? MediumCfg::LAYER_CAP : -1, m1, 2 * MediumCfg::LAYER_CAP, m2, s1, s2);
+    sieve_triples<EMIT, true>(j, w, w.pend[wp], lane, c, sb.B, e, s, s1, s2, w.left[0], m0, l1, m1, w.left[2], m2, wp,
+                              MediumTile::WARPS, sink, all, crowded, rows, np);
     return 0;
 }
 
@@ -2293,7 +2407,7 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
             const int n0 = w.off[3 * s + 1] - o0, n1 = w.off[3 * s + 2] - o0 - n0, n2 = w.off[3 * s + 3] - o0 - n0 - n1;
 #pragma unroll 1
             for (int ti = wp; ti < nT; ti += MediumTile::WARPS) {  // (CHAIN only: PAPER has one station)
-                if (!w.alive[ti]) continue;
+                if (!uniform(w.alive[ti])) continue;  // (uniform: see RowLists)
                 const float2 m = w.T[ti];
                 const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, shift3(w.sh, s), m.x, m.y,
                                               kStream ? w.Tt[ti] : make_float2(0.f, 0.f));

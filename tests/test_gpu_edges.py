@@ -135,3 +135,44 @@ def test_wide_windows_keep_their_speed(lib, S, n, narrow, wide, mode):
     b = _random_batch(6400000 // n // S, S, n, 5)
     t = [_time_us(_selection(lib, b, S, mode, w)) for w in (narrow, wide)]
     assert t[1] < 2.5 * t[0], t
+
+
+@pytest.mark.parametrize("n", [3, 13, 33, 64, 100, 128, 200, 300])
+def test_a_hit_far_from_the_others(lib, oracle_mod, n):
+    # one hit, or a whole straight track, at a huge slope or a small z, in every layer
+    # in turn, in the event itself or in its neighbours, whose hits lie behind it
+    rng = np.random.default_rng(200 + n)
+    zl = layer_z(2)
+    events = []
+    for slope, scale in ((1e3, 1.0), (1e5, 1.0), (-3e7, 1.0), (0.3, 0.3), (0.3, 0.01), (20.0, 0.1), (0.2, 50.0)):
+        for layer in range(7):
+            ev = []
+            for l, z in enumerate(zl):
+                s = rng.uniform(-0.4, 0.4, (n, 2))
+                hits = list(zip(s[:, 0] * z, s[:, 1] * z, np.full(n, z)))
+                track = [(0.1 * z + dx, 0.2 * z, z) for dx in (0.0, 0.05)]  # passes
+                if layer in (l, 6):  # 6: in every layer, so that the far hits pass as well
+                    zz = z * scale
+                    track.append((slope * zz, 0.5 * slope * zz, zz))
+                at = rng.integers(n + 1)
+                ev.append(hits[:at] + track + hits[at:])
+            events += [ev, [[(0.1 * z, 0.2 * z, z)] * (l % 3) for l, z in enumerate(zl)]]
+    b = make_batch(events, 2)
+    _oracle_same(lib, oracle_mod, b, 2, 0.01, record_caps=(-1, 0), label=f"n={n}")
+
+
+@pytest.mark.parametrize("slope,scale", [(1e5, 1.0), (None, 0.01)])
+@pytest.mark.parametrize("n,layer", [(20, 0), (60, 0), (60, 1), (60, 2), (200, 0), (200, 2)])
+def test_a_far_hit_keeps_the_speed(lib, n, layer, slope, scale):
+    # the first hit of every other event: its own station gets wide bounds for two
+    # pairs of layers (up to about 5 times the time of ordinary events), its
+    # neighbours none.  One bound for the station took 20 to 200 times.
+    b = _random_batch(400000 // n, 4, n, 6)
+    usual = _time_us(_selection(lib, b, 4, 1, 0.5))
+    first = b["offsets"][layer:-1:12][::2]
+    if slope:
+        b["x"][first] = slope * b["z"][first]
+    for a in ("x", "y", "z"):
+        b[a][first] *= np.float32(scale)
+    far = _time_us(_selection(lib, b, 4, 1, 0.5))
+    assert far < 8.0 * usual, (usual, far)
