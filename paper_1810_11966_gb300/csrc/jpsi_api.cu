@@ -844,6 +844,7 @@ jpsi_status run_host_pipelined(jpsi_ctx* c, RunState& rs, const jpsi_batch* hb, 
         Job jk = all;  // the chunk's events
         jk.ev_begin = e0;
         jk.ev_count = e1 - e0;
+        jk.n_src = hoff[e1 * S3];  // the hits behind are still being copied (or filled)
         if ((e = cudaStreamWaitEvent(st, rs.chunk_ev[k], 0)) != cudaSuccess ||
             (ztable && (e = launch_expand_z((const int32_t*)c->hoff.p, (const float*)rs.ztab.p, (float*)c->hz.p, e0,
                                             e1, (int)S, hb->n_hits, c->n_sm, st)) != cudaSuccess) ||

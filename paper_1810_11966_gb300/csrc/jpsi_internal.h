@@ -87,7 +87,10 @@ struct Job {
     const int32_t* off;
     int64_t n_events;             // events of the whole batch
     int64_t n_hits;               // hits of the batch (its last offset)
-    int64_t n_src;                // hits in the arrays
+    // Hits in the arrays.  The warp path reads whole rounds, so up to 191 hits behind a
+    // station, but none from n_src on; what lies there otherwise (another event's hits)
+    // only widens bounds or asks for the exact classification, never changes a result.
+    int64_t n_src;
     int64_t ev_begin, ev_count;   // events the warp kernels take from the batch (all by default)
     int32_t S, trig, mode, minc;
     int32_t distinct;             // distinct_hits: accept bits from dpair when minc == 2

@@ -176,3 +176,31 @@ def test_a_far_hit_keeps_the_speed(lib, n, layer, slope, scale):
         b[a][first] *= np.float32(scale)
     far = _time_us(_selection(lib, b, 4, 1, 0.5))
     assert far < 8.0 * usual, (usual, far)
+
+
+def _host_run(lib, ctx, b, S):
+    n = b["n_events"]
+    out = {"accept_bits": np.zeros((n + 31) // 32, np.uint32), "track_counts": np.zeros(n, np.int32),
+           "trip_off": np.zeros(n * S + 1, np.int64), "triplets": None}
+    o = lib.jpsi_outputs()
+    o.accept_bits, o.track_counts = out["accept_bits"].ctypes.data, out["track_counts"].ctypes.data
+    o.trip_off = out["trip_off"].ctypes.data
+    hb = lib.make_batch(b["x"], b["y"], b["z"], b["offsets"], n)
+    out["status"] = lib.jpsi_run_host(ctx.ctx, hb, o, 0)
+    out["trip_needed"] = o.trip_needed
+    return out
+
+
+def test_chunked_host_run_over_old_hits(lib):
+    # the device buffers hold another batch's odd coordinates where the chunks that
+    # are not copied yet will go: the stations before them are as they are alone
+    from gpu_helpers import assert_same
+    b = _random_batch(140_000, 1, 5, 7, r_max=0.12)
+    odd = dict(b, x=np.full_like(b["x"], np.nan), y=np.full_like(b["y"], 1e38))
+    ctx = lib.Context(lib.params(1, 1, t_xz=4.0, t_yz=4.0))
+    assert _host_run(lib, ctx, odd, 1)["status"] == 0
+    got = _host_run(lib, ctx, b, 1)
+    ref = gpu_select(ctx, b, triplets=False)
+    assert ref["trip_needed"] > 1000
+    assert_same(got, ref, b["n_events"], check_triplets=False)
+    ctx.close()
