@@ -777,9 +777,11 @@ jpsi_status run_host_pipelined(jpsi_ctx* c, RunState& rs, const jpsi_batch* hb, 
     int64_t cs = (ne + nch - 1) / nch;
     cs = (cs + 31) / 32 * 32;  // whole accept-bit words per chunk
     const int32_t* hoff = hb->offsets;
+    int64_t before = 0;
     for (int64_t e = 0; e <= ne; e += cs) {  // chunk boundaries must be usable as copy ranges
-        const int64_t b = hoff[std::min(e, ne) * S3];
-        if (b < 0 || b > hb->n_hits) return JPSI_EBUSY;
+        const int64_t b = hoff[e * S3];
+        if (b < before || b > hb->n_hits) return JPSI_EBUSY;
+        before = b;
     }
     if (hoff[ne * S3] != hb->n_hits) return JPSI_EBUSY;
     jpsi_status s;

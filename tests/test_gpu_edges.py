@@ -204,3 +204,18 @@ def test_chunked_host_run_over_old_hits(lib):
     assert ref["trip_needed"] > 1000
     assert_same(got, ref, b["n_events"], check_triplets=False)
     ctx.close()
+
+
+def test_chunk_boundaries_that_fall(lib):
+    # the third chunk's first offset lies before the second's: no copy range comes
+    # from it, and the batch is refused as malformed
+    n = 200_000
+    b = _random_batch(n, 1, 1, 8)
+    chunks = n // 65536
+    step = (-(-n // chunks) + 31) // 32 * 32
+    off = b["offsets"].copy()
+    off[3 * step * 2] = 3
+    ctx = lib.Context(lib.params(1, 1, t_xz=0.25))
+    assert _host_run(lib, ctx, dict(b, offsets=off), 1)["status"] == lib.JPSI_EINVAL
+    assert _host_run(lib, ctx, b, 1)["status"] == 0
+    ctx.close()
