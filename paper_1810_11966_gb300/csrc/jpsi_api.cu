@@ -258,19 +258,22 @@ float pruning_K(float cx, float cy) {
     return f;
 }
 
-bool device_accessible(jpsi_ctx* c, const void* p) {
+// Can the device read p?  `host` (if given) is set when p is host memory, read over
+// the link.
+bool device_accessible(jpsi_ctx* c, const void* p, bool* host = nullptr) {
     if (!p) return true;
     cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return c->pageable_ok;
-    }
-    if (a.type == cudaMemoryTypeDevice) return a.device == c->device;
-    if (a.type == cudaMemoryTypeManaged || a.type == cudaMemoryTypeHost) return true;
-    return c->pageable_ok;
+    const bool known = cudaPointerGetAttributes(&a, p) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    if (known && a.type == cudaMemoryTypeDevice) return a.device == c->device;
+    if (known && a.type == cudaMemoryTypeManaged) return true;
+    if (host) *host = true;
+    return (known && a.type == cudaMemoryTypeHost) || c->pageable_ok;
 }
 
-jpsi_status check_batch(jpsi_ctx* c, const jpsi_batch* b, const jpsi_outputs* o, bool device_ptrs) {
+// `host_hits` (if given): the hits, or some of them, are in host memory.
+jpsi_status check_batch(jpsi_ctx* c, const jpsi_batch* b, const jpsi_outputs* o, bool device_ptrs,
+                        bool* host_hits = nullptr) {
     if (!b || !o) return fail(c, JPSI_EINVAL, "null batch or outputs");
     const int64_t S = c->p.n_stations;
     if (b->n_events < 0 || b->n_hits < 0) return fail(c, JPSI_EINVAL, "negative sizes");
@@ -282,8 +285,10 @@ jpsi_status check_batch(jpsi_ctx* c, const jpsi_batch* b, const jpsi_outputs* o,
     if (o->triplets && !o->trip_off) return fail(c, JPSI_EINVAL, "triplets need trip_off");
     if (o->trip_capacity < 0) return fail(c, JPSI_EINVAL, "negative triplet capacity");
     if (device_ptrs) {
-        const void* ptrs[] = {b->x, b->y, b->z, b->offsets, b->z_layer, o->accept_bits, o->track_counts, o->trip_off,
-                              o->triplets};
+        const void* hits[] = {b->x, b->y, b->z};
+        for (const void* p : hits)
+            if (!device_accessible(c, p, host_hits)) return fail(c, JPSI_EINVAL, "pointer is not device-accessible");
+        const void* ptrs[] = {b->offsets, b->z_layer, o->accept_bits, o->track_counts, o->trip_off, o->triplets};
         for (const void* p : ptrs)
             if (!device_accessible(c, p)) return fail(c, JPSI_EINVAL, "pointer is not device-accessible");
     }
@@ -1088,9 +1093,10 @@ jpsi_status jpsi_run_plain(jpsi_ctx* c, const jpsi_batch* b, jpsi_outputs* o, vo
     if (!g.ok) return fail(c, JPSI_EBUSY, "context in use");
     cudaSetDevice(c->device);
     c->last_error.clear();
-    jpsi_status s = check_batch(c, b, o, true);
+    bool host_hits = false;
+    jpsi_status s = check_batch(c, b, o, true, &host_hits);
     if (s != JPSI_OK) return s;
-    return run_device(c, c->rs, b, o, (cudaStream_t)stream, false);
+    return run_device(c, c->rs, b, o, (cudaStream_t)stream, false, host_hits);
 }
 
 jpsi_status jpsi_run(jpsi_ctx* c, const jpsi_batch* b, jpsi_outputs* o, void* stream) {
@@ -1100,9 +1106,10 @@ jpsi_status jpsi_run(jpsi_ctx* c, const jpsi_batch* b, jpsi_outputs* o, void* st
     if (!g.ok) return fail(c, JPSI_EBUSY, "context in use");
     cudaSetDevice(c->device);
     c->last_error.clear();
-    jpsi_status s = check_batch(c, b, o, true);
+    bool host_hits = false;
+    jpsi_status s = check_batch(c, b, o, true, &host_hits);
     if (s != JPSI_OK) return s;
-    return run_device(c, c->rs, b, o, (cudaStream_t)stream, true);
+    return run_device(c, c->rs, b, o, (cudaStream_t)stream, true, host_hits);
 }
 
 jpsi_status jpsi_run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, void* stream) {

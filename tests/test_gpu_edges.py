@@ -219,3 +219,27 @@ def test_chunk_boundaries_that_fall(lib):
     assert _host_run(lib, ctx, dict(b, offsets=off), 1)["status"] == lib.JPSI_EINVAL
     assert _host_run(lib, ctx, b, 1)["status"] == 0
     ctx.close()
+
+
+def test_run_on_pinned_hits(lib, oracle_mod):
+    # hits in pinned memory are read over the link, each once: full rounds of a warp
+    # read up to four times as many (1.4 times the one-launch form's time, where
+    # events come one by one; 1.15 without them)
+    import torch
+    b = _random_batch(20_000, 4, 5, 9)
+    d = {k: torch.from_numpy(b[k]).pin_memory() for k in ("x", "y", "z")}
+    off = torch.from_numpy(b["offsets"]).cuda()
+    ctx = lib.Context(lib.params(4, 1, t_xz=0.25, t_yz=0.25))
+    tracks = torch.zeros(b["n_events"], dtype=torch.int32, device="cuda")
+    o = lib.jpsi_outputs()
+    o.track_counts = tracks.data_ptr()
+    hb = lib.make_batch(d["x"], d["y"], d["z"], off, b["n_events"])
+    t = {}
+    for call in (lib.jpsi_run, lib.jpsi_run_plain):
+        def f():
+            assert call(ctx.ctx, hb, o, torch.cuda.current_stream().cuda_stream) == 0
+        t[call] = _time_us(f)
+    ref = oracle_mod.run(oracle_mod.params(4, 1, t_xz=0.25), b, n_threads=8)
+    assert np.array_equal(tracks.cpu().numpy(), ref["track_counts"])
+    assert t[lib.jpsi_run] < 1.28 * t[lib.jpsi_run_plain], t
+    ctx.close()
