@@ -190,8 +190,13 @@ jpsi_status jpsi_run_host(jpsi_ctx *ctx, const jpsi_batch *batch, jpsi_outputs *
  * (i, j, k) of unit w*S + s names hits offsets[3s] + i, offsets[3s+1] + j,
  * offsets[3s+2] + k of the timeslice.  All pointers are device memory.  The
  * library builds one event per window on the device (its hits within the
- * window's time range, read where they are), so the budget must hold about 80
- * bytes per window and station, and 4 per hit with z_layer.  JPSI_EINVAL for a
+ * window's time range, read where they are).  The budget must hold, for K
+ * windows of S stations: 72 K S + 40 K bytes (ranges, offsets, counts, lists);
+ * 17 P for the P = min(max(64 K, 65 536), 2^24) entries of the trigger pool;
+ * 557 056 per block of the block tile, of which a GPU runs up to three per SM
+ * (254 MB on 152 SMs); with z_layer 4 bytes per hit of the timeslice or 16 per
+ * hit of the windows' ranges, whichever is less.  A triplet record is kept on
+ * top where the budget has room for it.  JPSI_EINVAL for a
  * malformed timeslice (the time order, NaN times, z <= 0 and the bounds are
  * checked on the device), for distinct_hits = 1, and when the windows'
  * ranges hold 2^31 hits or more (split the timeslice).  jpsi_run_stream runs

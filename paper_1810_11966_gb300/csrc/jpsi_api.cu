@@ -156,8 +156,9 @@ struct jpsi_ctx {
     RunState rs;
     // device copies for jpsi_run_host
     DevBuf hx, hy, hz, hoff, hacc, htc, htoff, htrip;
-    // window batch of a free-streaming run: ranges, their scan, offsets, places; z from a table
-    DevBuf wlo, wcnt, woff, wbs, woff32, wshift, wz;
+    // window batch of a free-streaming run: ranges, their scan, offsets; z from a table,
+    // or copies of the windows' hits
+    DevBuf wlo, wcnt, woff, wbs, woff32, wx, wy, wz, wt;
     std::string last_error;
     std::mutex err_mu, cap_mu, alloc_mu;
     std::atomic<bool> timing{false};
@@ -901,7 +902,7 @@ jpsi_status run_host_pipelined(jpsi_ctx* c, RunState& rs, const jpsi_batch* hb, 
 }
 
 // A free-streaming timeslice: windows become the events of a window batch
-// (ranges found and gathered on the device), the selection runs with the
+// (ranges found on the device, their hits read in place), the selection runs with the
 // time tests compiled in, and the triplet rows are moved back to timeslice
 // group indices.
 jpsi_status run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, cudaStream_t st, bool batched) {
@@ -935,9 +936,7 @@ jpsi_status run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, c
         (s = ensure(c, c->wcnt, (size_t)std::max<int64_t>(n, 1) * 4, "window ranges")) ||
         (s = ensure(c, c->woff, (size_t)(n + 1) * 8, "window ranges")) ||
         (s = ensure(c, c->wbs, (size_t)((n + 4095) / 4096 + 1) * 8, "scan")) ||
-        (s = ensure(c, c->woff32, (size_t)(n + 1) * 4, "window offsets")) ||
-        (s = ensure(c, c->wshift, (size_t)std::max<int64_t>(n, 1) * 4, "window places")) ||
-        (!ts->z && (s = ensure(c, c->wz, (size_t)std::max<int64_t>(ts->n_hits, 1) * 4, "hits z"))))
+        (s = ensure(c, c->woff32, (size_t)(n + 1) * 4, "window offsets")))
         return s;
     RunState& rs = c->rs;
     WinJob w{};
@@ -959,7 +958,6 @@ jpsi_status run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, c
     w.woff = (int64_t*)c->woff.p;
     w.block_sums = (int64_t*)c->wbs.p;
     w.off_out = (int32_t*)c->woff32.p;
-    w.shift = (int32_t*)c->wshift.p;
     w.ctrl = rs.d_ctrl;
     w.n_sm = c->n_sm;
     const bool timing = c->timing.load();
@@ -974,11 +972,6 @@ jpsi_status run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, c
     const int64_t total = rs.h_ctrl->trip_total;
     if (total >= ((int64_t)1 << 31))
         return fail(c, JPSI_EINVAL, "the windows' hit ranges hold 2^31 hits or more: split the timeslice");
-    const bool fill_z = !ts->z && ts->n_hits > 0;
-    if ((e = streamk::launch_window_place(w, st)) != cudaSuccess) return cuda_fail(c, e, "window places");
-    if (fill_z && (e = streamk::launch_window_z(w, (float*)c->wz.p, st)) != cudaSuccess)
-        return cuda_fail(c, e, "z from geometry");
-    if (timing) cudaEventRecord(rs.ev[6], st);
     // windows in place of events: their offsets count the hits, the hits stay
     // where they are
     jpsi_batch wbat{};
@@ -986,12 +979,37 @@ jpsi_status run_stream(jpsi_ctx* c, const jpsi_timeslice* ts, jpsi_outputs* o, c
     wbat.n_hits = total;
     wbat.x = ts->x;
     wbat.y = ts->y;
-    wbat.z = ts->z ? ts->z : (const float*)c->wz.p;
+    wbat.z = ts->z;
     wbat.offsets = w.off_out;
-    const StreamJob sj{ts->t, ts->bounds, ts->dt, w.shift, ts->n_hits};
+    StreamJob sj{ts->t, ts->bounds, ts->dt, w.wcnt, ts->n_hits};
+    const bool fill_z = !ts->z && ts->n_hits > 0;
+    // z from a table: of every hit of the timeslice (4 bytes), or, where the windows
+    // hold less than a quarter of them, in copies of the windows' hits (16 bytes),
+    // which need less memory then (and less time: one window of a 120 M-hit
+    // timeslice 481 -> 360 us, 10 000 of them 760 -> 710)
+    const bool gather = fill_z && total <= ts->n_hits / 4;
+    if (gather) {
+        const size_t hb = (size_t)std::max<int64_t>(total, 1) * 4;
+        if ((s = ensure(c, c->wx, hb, "window hits")) || (s = ensure(c, c->wy, hb, "window hits")) ||
+            (s = ensure(c, c->wz, hb, "window hits")) || (s = ensure(c, c->wt, hb, "window hits")))
+            return s;
+        wbat.x = w.xo = (float*)c->wx.p;
+        wbat.y = w.yo = (float*)c->wy.p;
+        w.zo = (float*)c->wz.p;
+        sj.t = w.to = (float*)c->wt.p;
+        if ((e = streamk::launch_window_gather(w, st)) != cudaSuccess) return cuda_fail(c, e, "window gather");
+        sj.n_src = total;
+    } else {
+        if ((e = streamk::launch_window_place(w, st)) != cudaSuccess) return cuda_fail(c, e, "window places");
+        if (fill_z && ((s = ensure(c, c->wz, (size_t)ts->n_hits * 4, "hits z")) != JPSI_OK)) return s;
+        if (fill_z && (e = streamk::launch_window_z(w, (float*)c->wz.p, st)) != cudaSuccess)
+            return cuda_fail(c, e, "z from geometry");
+    }
+    if (fill_z) wbat.z = (const float*)c->wz.p;
+    if (timing) cudaEventRecord(rs.ev[6], st);
     s = run_device(c, rs, &wbat, o, st, batched, false, kStreamL, &sj);
     if (s != JPSI_OK) return s;
-    int launches = kLaunchesWindows + (fill_z ? 1 : 0);
+    int launches = kLaunchesWindows + (fill_z && !gather ? 1 : 0);
     const bool rows = o->triplets && o->trip_needed > 0;
     if (rows) {
         if (timing) cudaEventRecord(rs.ev[7], st);
@@ -1079,7 +1097,7 @@ void jpsi_destroy(jpsi_ctx* c) {
     cudaDeviceSynchronize();
     state_free(c, c->rs);
     DevBuf* bufs[] = {&c->hx,  &c->hy,   &c->hz,  &c->hoff, &c->hacc, &c->htc, &c->htoff, &c->htrip, &c->wlo,
-                      &c->wcnt, &c->woff, &c->wbs, &c->woff32, &c->wshift, &c->wz};
+                      &c->wcnt, &c->woff, &c->wbs, &c->woff32, &c->wx, &c->wy, &c->wz, &c->wt};
     for (DevBuf* b : bufs) release(c, *b);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);

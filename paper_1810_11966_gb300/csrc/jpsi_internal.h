@@ -206,24 +206,27 @@ struct WinJob {
     int32_t S, trig, chain;
     float dt;
     int32_t* wlo;          // [K*3S] first timeslice hit of each range
-    int32_t* wcnt;         // [K*3S] hits of each range
+    int32_t* wcnt;         // [K*3S] hits of each range; then how far its hits lie from off_out's places
     int64_t* woff;         // [K*3S + 1] exclusive scan of wcnt
     int64_t* block_sums;   // scan scratch
     int32_t* off_out;      // [K*3S + 1] the window batch's offsets
-    int32_t* shift;        // [K*3S] from them to the timeslice's hits
+    float *xo, *yo, *zo, *to;  // copies of the windows' hits (launch_window_gather)
     Ctrl* ctrl;            // status (kStInvalid) and trip_total = the window batch's hits
     int n_sm;
 };
 namespace streamk {
 //   launch_window_ranges: validates the timeslice (times sorted per group, no
 //     NaN; z > 0 where read; bounds finite and increasing), finds each
-//     window's ranges and scans their sizes (4 launches).
+//     window's ranges and scans their sizes (5 launches).
 //   launch_window_place: the window batch's offsets and its hits' places (1 launch).
+//   launch_window_gather: the offsets, and the windows' hits copied to them, z from
+//     the table (1 launch, in place of launch_window_place).
 //   launch_window_z: per-hit z of the timeslice from its table (1 launch).
 //   launch_window_rows: triplet rows from window-batch indices to timeslice
 //     layer-group indices (1 launch).
 cudaError_t launch_window_ranges(const WinJob& w, cudaStream_t st);
 cudaError_t launch_window_place(const WinJob& w, cudaStream_t st);
+cudaError_t launch_window_gather(const WinJob& w, cudaStream_t st);
 cudaError_t launch_window_z(const WinJob& w, float* z, cudaStream_t st);
 cudaError_t launch_window_rows(const WinJob& w, const int64_t* trip_off, int32_t* triplets, cudaStream_t st);
 }  // namespace streamk

@@ -3573,8 +3573,30 @@ __global__ void __launch_bounds__(256) k_win_place(const __grid_constant__ WinJo
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q <= n; q += stride) {
         const int64_t at = w.woff[q];
         w.off_out[q] = (int32_t)at;
-        if (q < n) w.shift[q] = (int32_t)(w.wlo[q] - at);
+        if (q < n) w.wcnt[q] = (int32_t)(w.wlo[q] - at);  // (the sizes are in the scan)
     }
+}
+
+// The window batch of few windows of a large timeslice without per-hit z: its
+// offsets, and its hits copied there, one warp per (window, group) range.
+__global__ void __launch_bounds__(256) k_win_gather(const __grid_constant__ WinJob w) {
+    const int S3 = 3 * w.S, lane = threadIdx.x & 31;
+    const int64_t n = w.K * S3, nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < n; q += nwarps) {
+        const int64_t at = w.woff[q], lo = w.wlo[q], cnt = w.woff[q + 1] - at;
+        const float v = __ldg(w.z_layer + (int)(q % S3));
+        if (lane == 0) {
+            w.off_out[q] = (int32_t)at;
+            w.wcnt[q] = 0;
+        }
+        for (int64_t i = lane; i < cnt; i += 32) {
+            w.xo[at + i] = __ldg(w.x + lo + i);
+            w.yo[at + i] = __ldg(w.y + lo + i);
+            w.to[at + i] = __ldg(w.t + lo + i);
+            w.zo[at + i] = v;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) w.off_out[n] = (int32_t)w.woff[n];
 }
 
 // Per-hit z of the timeslice from the per-group table.
@@ -3639,6 +3661,11 @@ cudaError_t launch_window_ranges(const WinJob& w, cudaStream_t st) {
 
 cudaError_t launch_window_place(const WinJob& w, cudaStream_t st) {
     k_win_place<<<win_grid(w.K * 3 * w.S + 1, w.n_sm), 256, 0, st>>>(w);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_window_gather(const WinJob& w, cudaStream_t st) {
+    k_win_gather<<<win_grid(w.K * 3 * w.S * 32, w.n_sm), 256, 0, st>>>(w);
     return cudaGetLastError();
 }
 

@@ -243,3 +243,59 @@ def test_run_on_pinned_hits(lib, oracle_mod):
     assert np.array_equal(tracks.cpu().numpy(), ref["track_counts"])
     assert t[lib.jpsi_run] < 1.28 * t[lib.jpsi_run_plain], t
     ctx.close()
+
+
+def _timeslice(n_groups_hits, K, dt, seed):
+    """A timeslice of two stations on the device: `n_groups_hits` hits in each layer, times
+    uniform over 1 s of ns, and K windows of 1 us at its middle."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    n = n_groups_hits
+    zl = torch.tensor(layer_z(2), dtype=torch.float32, device="cuda")
+    t = torch.sort(torch.rand(6, n, generator=g, device="cuda") * 1e9, dim=1)[0].reshape(-1).contiguous()
+    z = zl.repeat_interleave(n)
+    s = torch.rand(2, 6 * n, generator=g, device="cuda") * 0.02
+    off = torch.arange(7, dtype=torch.int32, device="cuda") * n
+    # windows of 8 us (64 ns is the spacing of floats at 5e8): about 16 hits per layer
+    bounds = 5e8 + 8192.0 * torch.arange(K + 1, dtype=torch.float32, device="cuda")
+    return {"x": (s[0] * z).contiguous(), "y": (s[1] * z).contiguous(), "z": z, "t": t, "offsets": off, "zl": zl,
+            "bounds": bounds, "dt": dt}
+
+
+def _stream_run(lib, ts, table, budget=0):
+    import torch
+    K = len(ts["bounds"]) - 1
+    ctx = lib.Context(lib.params(2, 1, t_xz=0.04, t_yz=0.04), hbm_budget=budget)
+    out = [torch.zeros(m, dtype=d, device="cuda") for m, d in (((K + 31) // 32, torch.int32), (K, torch.int32),
+                                                               (2 * K + 1, torch.int64))]
+    o = lib.jpsi_outputs()
+    o.accept_bits, o.track_counts, o.trip_off = (a.data_ptr() for a in out)
+    t = lib.make_timeslice(ts["x"], ts["y"], None if table else ts["z"], ts["t"], ts["offsets"], ts["bounds"], ts["dt"],
+                           z_layer=ts["zl"] if table else None)
+    status = lib.jpsi_run_stream(ctx.ctx, t, o, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    ctx.close()
+    return status, o.trip_needed, [a.cpu().numpy() for a in out]
+
+
+@pytest.mark.parametrize("K", [1, 5, 3000, 20000])
+def test_windows_of_a_large_timeslice_by_z_table(lib, K):
+    # few windows: copies of their hits, not z for every hit of the timeslice; many: z
+    # filled in.  The budget is the documented one, and the results are those of per-hit z
+    import torch
+    ts = _timeslice(2_000_000, K, 4096.0, K)
+    per_hit = _stream_run(lib, ts, False)
+    assert per_hit[0] == 0 and (K < 100 or per_hit[1] > 0)
+    n_hits = len(ts["x"])
+    # every window's range is at most its width and four dt
+    ranges = 6 * K * (2_000_000 * (8192.0 + 5 * 4096.0) / 1e9 * 1.5 + 40)
+    props = torch.cuda.get_device_properties(0)
+    budget = (72 * K * 2 + 40 * K + 17 * min(max(64 * K, 65536), 1 << 24) + 557056 * 3 * props.multi_processor_count
+              + int(min(4 * n_hits, 16 * ranges)) + 4096)
+    got = _stream_run(lib, ts, True, budget)
+    assert got[0] == 0, budget
+    assert got[1] == per_hit[1]
+    for a, b in zip(got[2], per_hit[2]):
+        assert np.array_equal(a, b)
+    # a budget below the fixed part is refused, not overrun
+    assert _stream_run(lib, ts, True, budget // 3)[0] == lib.JPSI_ENOMEM
