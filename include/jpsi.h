@@ -218,7 +218,9 @@ jpsi_status jpsi_run_stream_plain(jpsi_ctx *ctx, const jpsi_timeslice *ts, jpsi_
  * (its one kernel has one thread per event, Sec. 5.3); none of these knobs
  * changes a result.
  *   light_wpb          warps per block of the small warp-tile kernel: 2, 4 or 8.
- *   light_grab         events a persistent warp takes per atomic grab: 1 .. 64.
+ *   light_grab         events a persistent warp takes per atomic grab, at most:
+ *                      1 .. 64 (fewer in batches that have not two such grabs
+ *                      for every resident warp).
  *   small_layer_cap    most hits in any layer of a processed station for an
  *                      event to stay on the small warp tile: 1 .. 192.
  *   medium_layer_cap   the same for the medium warp tile: 1 .. 384; events

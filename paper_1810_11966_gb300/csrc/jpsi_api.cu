@@ -296,6 +296,13 @@ jpsi_status check_batch(jpsi_ctx* c, const jpsi_batch* b, const jpsi_outputs* o,
     return JPSI_OK;
 }
 
+// Events per grab in a batch of ne: one until every resident warp has two grabs (64
+// events, two warps' worth of the default grab, took twice an event's time).
+int32_t events_per_grab(const jpsi_ctx* c, int64_t ne) {
+    const int64_t warps = (int64_t)c->batch_cfg.light_blocks * c->batch_cfg.light_wpb;
+    return (int32_t)std::max<int64_t>(1, std::min<int64_t>(c->tune.light_grab, ne / (2 * std::max<int64_t>(warps, 1))));
+}
+
 // Prepares scratch and the job descriptor of a run.
 jpsi_status prepare(jpsi_ctx* c, RunState& rs, const jpsi_batch* b, jpsi_outputs* o, bool host_hits,
                     bool stream = false) {
@@ -349,10 +356,7 @@ jpsi_status prepare(jpsi_ctx* c, RunState& rs, const jpsi_batch* b, jpsi_outputs
     j.cx = c->cx;
     j.cy = c->cy;
     j.K = c->K;
-    // events per grab: one until every resident warp has two grabs (64 events,
-    // two warps' worth of the default grab, took twice an event's time)
-    const int64_t warps = (int64_t)c->batch_cfg.light_blocks * c->batch_cfg.light_wpb;
-    j.grab = (int32_t)std::max<int64_t>(1, std::min<int64_t>(c->tune.light_grab, ne / (2 * std::max<int64_t>(warps, 1))));
+    j.grab = events_per_grab(c, ne);
     j.cap_small = c->tune.small_layer_cap;
     j.cap_medium = c->tune.medium_layer_cap;
     j.host_hits = host_hits ? 1 : 0;
@@ -1276,10 +1280,18 @@ jpsi_status jpsi_autotune(jpsi_ctx* c, const jpsi_batch* sample) {
     // one dimension at a time, each from the best shape so far
     for (int w : {2, 4, 8}) {
         if (light_max_blocks_per_sm(w) < 1) continue;
-        for (int gr : {1, 2, 4, 8}) {
+        // grabs that the sample is too small to tell from one tried before (the
+        // context's own comes first) are not tried: the winner would be chance
+        uint64_t tried = 0;  // bit g - 1: g events per grab
+        for (int gr : {start.light_grab, 1, 2, 4, 8}) {
             jpsi_tuning t = best;
             t.light_wpb = w;
             t.light_grab = gr;
+            c->tune = t;
+            apply_tuning(c);
+            const uint64_t bit = 1ull << (events_per_grab(c, sample->n_events) - 1);
+            if (tried & bit) continue;
+            tried |= bit;
             trial(t);
         }
     }

@@ -299,3 +299,18 @@ def test_windows_of_a_large_timeslice_by_z_table(lib, K):
         assert np.array_equal(a, b)
     # a budget below the fixed part is refused, not overrun
     assert _stream_run(lib, ts, True, budget // 3)[0] == lib.JPSI_ENOMEM
+
+
+@pytest.mark.parametrize("grab", [1, 3, 8, 64])
+def test_autotune_keeps_a_grab_it_cannot_measure(lib, grab):
+    # 500 events are one per grab whatever the limit: no limit is better than another
+    import torch
+    b = _random_batch(500, 4, 20, 10)
+    ctx = lib.Context(lib.params(4, 1, t_xz=0.25))
+    tu = lib.jpsi_get_tuning(ctx.ctx)
+    tu.light_grab = grab
+    assert lib.jpsi_set_tuning(ctx.ctx, tu) == lib.JPSI_OK
+    d = {k: torch.from_numpy(b[k]).cuda() for k in ("x", "y", "z", "offsets")}
+    assert lib.jpsi_autotune(ctx.ctx, lib.make_batch(d["x"], d["y"], d["z"], d["offsets"], 500)) == 0
+    assert lib.jpsi_get_tuning(ctx.ctx).light_grab == grab
+    ctx.close()
