@@ -314,3 +314,86 @@ def test_autotune_keeps_a_grab_it_cannot_measure(lib, grab):
     assert lib.jpsi_autotune(ctx.ctx, lib.make_batch(d["x"], d["y"], d["z"], d["offsets"], 500)) == 0
     assert lib.jpsi_get_tuning(ctx.ctx).light_grab == grab
     ctx.close()
+
+
+def _tiled(rng, n_events, n_base=61):
+    """n_events events of one station, the same n_base over and over; the counts' period."""
+    base = make_batch([[[(0.1 * z + rng.normal(0, 0.1), 0.2 * z, z) for _ in range(rng.integers(0, 5))]
+                        for z in layer_z(1)] for _ in range(n_base)], 1)
+    cnt = np.resize(np.diff(base["offsets"]), 3 * n_events)
+    off = np.concatenate([[0], np.cumsum(cnt)]).astype(np.int32)
+    return base, {**{k: np.resize(base[k], off[-1]) for k in ("x", "y", "z")}, "offsets": off, "n_events": n_events,
+                  "n_hits": int(off[-1]), "n_stations": 1}
+
+
+@pytest.mark.parametrize("grab", [2, 4, 8])
+def test_events_per_grab_at_its_steps(lib, oracle_mod, grab):
+    # g events per grab from 2 W g events on, W warps resident: 28 an SM as built, and
+    # what other register counts would give
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(19)
+    ctx = lib.Context(lib.params(1, 1, t_xz=0.25))
+    tu = lib.jpsi_get_tuning(ctx.ctx)
+    tu.light_grab = grab
+    assert lib.jpsi_set_tuning(ctx.ctx, tu) == lib.JPSI_OK
+    base, _ = _tiled(rng, 1)
+    ref = oracle_mod.run(oracle_mod.params(1, 1, t_xz=0.25), base)
+    for warps in (24, 28, 32):
+        for n in (2 * warps * sms * grab + d for d in (-1, 0, 1, grab - 1)):
+            rng = np.random.default_rng(19)
+            _, b = _tiled(rng, n)
+            got = gpu_select(ctx, b, triplets=False)
+            assert got["status"] == 0
+            assert np.array_equal(got["track_counts"], np.resize(ref["track_counts"], n)), (warps, n)
+    ctx.close()
+
+
+@pytest.mark.parametrize("warps", [24, 28, 32])
+def test_noalloc_grab_at_its_step(lib, oracle_mod, warps):
+    # two events per grab beyond 4 W events
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    p = lib.params(1, 1, t_xz=0.25)
+    for d in (-1, 0, 1, 2):
+        n = 4 * warps * sms + d
+        base, b = _tiled(np.random.default_rng(19), n)
+        ref = oracle_mod.run(oracle_mod.params(1, 1, t_xz=0.25), base)
+        t = {k: torch.from_numpy(b[k]).cuda() for k in ("x", "y", "z", "offsets")}
+        tracks, units = (torch.full((n,), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+        assert lib.jpsi_select_noalloc(p, lib.make_batch(t["x"], t["y"], t["z"], t["offsets"], n), tracks.data_ptr(),
+                                       units.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        assert np.array_equal(tracks.cpu().numpy(), np.resize(ref["track_counts"], n)), n
+
+
+@pytest.mark.parametrize("S", [10, 11, 16])
+@pytest.mark.parametrize("host", [False, True])
+def test_z_table_of_many_stations(lib, oracle_mod, S, host):
+    # more than 31 layers: the table's second group of layers
+    import torch
+    rng = np.random.default_rng(S)
+    sz = tuple(130.0 + 35.0 * s for s in range(S))
+    zl = layer_z(S, station_z=sz)
+    events = [[[(0.1 * z + rng.normal(0, 0.1), 0.2 * z, z) for _ in range(rng.integers(0, 6))] for z in zl]
+              for _ in range(40)]
+    b = make_batch(events, S)
+    ref = oracle_mod.run(oracle_mod.params(S, 1, t_xz=0.25), b, n_threads=8)
+    assert ref["trip_needed"] > 0
+    ctx = lib.Context(lib.params(S, 1, t_xz=0.25))
+    table = np.array(zl, np.float32)
+    tracks = np.zeros(40, np.int32)
+    o = lib.jpsi_outputs()
+    if host:
+        o.track_counts = tracks.ctypes.data
+        hb = lib.make_batch(b["x"], b["y"], None, b["offsets"], 40, z_layer=table)
+        assert lib.jpsi_run_host(ctx.ctx, hb, o, 0) == 0
+    else:
+        d = {k: torch.from_numpy(b[k]).cuda() for k in ("x", "y", "offsets")}
+        dt, dz = torch.from_numpy(tracks).cuda(), torch.from_numpy(table).cuda()
+        o.track_counts = dt.data_ptr()
+        db = lib.make_batch(d["x"], d["y"], None, d["offsets"], 40, z_layer=dz)
+        assert lib.jpsi_run(ctx.ctx, db, o, torch.cuda.current_stream().cuda_stream) == 0
+        tracks = dt.cpu().numpy()
+    assert np.array_equal(tracks, ref["track_counts"]) and o.trip_needed == ref["trip_needed"]
+    ctx.close()
