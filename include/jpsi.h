@@ -305,8 +305,8 @@ jpsi_status jpsi_inject_fault(jpsi_ctx *ctx, int kind, int count);
  * two int fields report the batched form's current launch shape (warps per
  * block and events per grab of the warp-per-event kernel, as chosen by
  * jpsi_autotune or the defaults 4 and 2).  window_ms: free-streaming runs'
- * event building (window ranges, their scan, the gather of the window
- * batch, and the mapping of triplet rows back to the timeslice). */
+ * event building (window ranges, their scan, the places or copies of their
+ * hits, and the mapping of triplet rows back to the timeslice). */
 typedef struct {
     int64_t runs;
     int64_t kernel_launches; /* kernels of this library launched by those runs */

@@ -19,8 +19,8 @@
 //     |s_i - s_j| <= b_i (1 - 5e-5) + b_j (1 - 5e-5),
 // so the FP32 test |fl(s_i - s_j)| <= fl(b_i + b_j) never rejects a pair that
 // belongs to a passing triplet (K's 1e-4 slack covers the error of r, kappa
-// the relative errors of s and eps |m|).  The tiles keep one bound per layer,
-// B_l = max of b over the layer's stored hits, and test against
+// the relative errors of s and eps |m|).  The block tile keeps one bound per layer,
+// B_l = max of b over the layer's stored hits, and tests against
 // fl(B_l + B_l') >= fl(b_i + b_j) (rounding is monotone); the hits of a
 // detector layer share its z, so B_l is b up to the small kappa term.  Hits with a non-finite coordinate
 // cannot pass P1 at all (Szz, Suz or a residual becomes Inf/NaN) and are
@@ -109,29 +109,6 @@ __device__ __forceinline__ HitPrep hit_prep(float x, float y, float z, float K) 
     h.b = __fadd_rn(__fadd_rn(__fmul_rn(K, iz), __fmul_rn(kKappa, h.l1)), kTau);
     // b finite implies s_x, s_y finite (b >= kappa |s|)
     h.wild = h.live & !((z >= 1.17549435e-38f) & (z < 8.50705917e+37f) & (h.b < INFINITY));
-    return h;
-}
-
-// Fast staging path: slopes and bound without the per-hit classification.
-// ok is exactly live && !wild && !zbad of hit_prep: z in the normal range
-// [2^-126, 2^126) excludes z <= 0, NaN and Inf, and a finite b implies finite
-// s_x, s_y, hence finite x, y.
-struct HitFast {
-    float sx, sy, b;
-    float r, l1;  // as in HitPrep
-    bool ok;
-};
-
-__device__ __forceinline__ HitFast hit_fast(float x, float y, float z, float K) {
-    HitFast h;
-    float iz;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(iz) : "f"(z));
-    h.sx = __fmul_rn(x, iz);
-    h.sy = __fmul_rn(y, iz);
-    h.r = iz;
-    h.l1 = __fadd_rn(fabsf(h.sx), fabsf(h.sy));
-    h.b = __fadd_rn(__fadd_rn(__fmul_rn(K, iz), __fmul_rn(kKappa, h.l1)), kTau);
-    h.ok = (z >= 1.17549435e-38f) & (z < 8.50705917e+37f) & (h.b < INFINITY);
     return h;
 }
 

@@ -263,8 +263,6 @@ __device__ __forceinline__ int f2key(float f) {
     return i >= 0 ? i : i ^ 0x7fffffff;
 }
 __device__ __forceinline__ float key2f(int k) { return __int_as_float(k >= 0 ? k : k ^ 0x7fffffff); }
-__device__ __forceinline__ float warp_min(float v) { return key2f(__reduce_min_sync(kFull, f2key(v))); }
-__device__ __forceinline__ float warp_max(float v) { return key2f(__reduce_max_sync(kFull, f2key(v))); }
 
 __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
 #pragma unroll
@@ -494,11 +492,7 @@ __device__ __forceinline__ Win cell_window(const TV& t, int l, float cx, float c
     const LayerMeta& m = t.meta[l];
     Win w;
     query_bins<TV::NX>(cx, Wx, m.lox, m.scx, w.x0, w.x1);
-    if constexpr (TV::NY > 1) {
-        query_bins<TV::NY>(cy, Wy, m.loy, m.scy, w.y0, w.y1);
-    } else {
-        w.y0 = w.y1 = 0;
-    }
+    query_bins<TV::NY>(cy, Wy, m.loy, m.scy, w.y0, w.y1);
     return w;
 }
 
@@ -533,13 +527,11 @@ __device__ __forceinline__ float layer_pair_bound(const TV& t, int a, int b, flo
 }
 
 // Where passing trigger triplets' slopes go (CHAIN mode, trigger station).
-// Warp path: a warp-local count; block path: a block-shared counter.
 struct TSink {
     bool on;
     float2* T;
     int cap;
-    int* sh_n;  // block-shared counter, or null
-    int n;      // warp-local counter when sh_n is null
+    int* sh_n;  // their number (block-shared)
     bool norec = false;  // a repeated enumeration: record no triplet entries
     unsigned long long* ijk = nullptr;  // distinct_hits: the triplets' packed hits beside T
     float2* tt = nullptr;               // free-streaming windows: their (min t, max t) beside T
@@ -556,14 +548,12 @@ struct Pending {
 
 // P1 on the triples of the lanes with `has` (layer-local hits ii, jj, kk of
 // the layers that start at base0, base1, base2) and what follows from a pass:
-// the triplet's rank in its unit (warp-local on the warp path, from a block-
-// shared counter on the block path), its row (emit pass), its slopes for the
+// the triplet's rank in its unit (from the block-shared counter), its row (emit pass), its slopes for the
 // trigger sink (CHAIN) and its entry in the scatter record.  All lanes call it.
 template <bool EMIT>
 __device__ __forceinline__ void fit_and_record(const Job& j, int lane, const Cuts& c, bool has, int32_t base0,
                                                int32_t base1, int32_t base2, int ii, int jj, int kk, TSink& ts,
-                                               int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag,
-                                               int& count) {
+                                               int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag) {
     bool ok = false;
     float mx = 0.f, my = 0.f;
     float2 tt = make_float2(0.f, 0.f);
@@ -582,12 +572,9 @@ __device__ __forceinline__ void fit_and_record(const Job& j, int lane, const Cut
     const unsigned mask = __ballot_sync(kFull, ok);
     if (mask) {
         const int rk = __popc(mask & lanemask_lt()), np = __popc(mask);
-        int base = count;
-        if (sh_rank) {
-            int b = 0;
-            if (lane == 0) b = atomicAdd(sh_rank, np);
-            base = __shfl_sync(kFull, b, 0);
-        }
+        int base = 0;
+        if (lane == 0) base = atomicAdd(sh_rank, np);
+        base = __shfl_sync(kFull, base, 0);
         if (EMIT && ok && base + rk < limit &&  // never past the unit's rows
             JPSI_IN(j.ctrl, (rows - j.triplets) / 3 + base + rk < j.trip_cap)) {
             int32_t* r = rows + 3 * (int64_t)(base + rk);
@@ -596,14 +583,9 @@ __device__ __forceinline__ void fit_and_record(const Job& j, int lane, const Cut
             r[2] = kk;
         }
         if (ts.on) {
-            int tb = ts.n;
-            if (ts.sh_n) {
-                int b = 0;
-                if (lane == 0) b = atomicAdd(ts.sh_n, np);
-                tb = __shfl_sync(kFull, b, 0);
-            } else {
-                ts.n += np;
-            }
+            int tb = 0;
+            if (lane == 0) tb = atomicAdd(ts.sh_n, np);
+            tb = __shfl_sync(kFull, tb, 0);
             if (ok && tb + rk < ts.cap) {
                 ts.T[tb + rk] = make_float2(mx, my);
                 if (ts.ijk) ts.ijk[tb + rk] = pack_ijk(ii, jj, kk);
@@ -623,15 +605,13 @@ __device__ __forceinline__ void fit_and_record(const Job& j, int lane, const Cut
                 j.tscr[b] = te;
             }
         }
-        count += np;
     }
 }
 
 // The same on tile positions pi, pj, pk of a staged block tile.
 template <bool EMIT, class TV>
 __device__ __forceinline__ void fit_tile(const Job& j, const TV& t, int lane, const Cuts& c, bool has, int pi, int pj,
-                                         int pk, TSink& ts, int32_t* rows, int limit, int64_t unit, int* sh_rank,
-                                         int tag, int& count) {
+                                         int pk, TSink& ts, int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag) {
     int ii = 0, jj = 0, kk = 0;
     if (has) {
         ii = t.idx[pi];
@@ -639,7 +619,7 @@ __device__ __forceinline__ void fit_tile(const Job& j, const TV& t, int lane, co
         kk = t.idx[pk];
     }
     fit_and_record<EMIT>(j, lane, c, has, t.meta[0].base, t.meta[1].base, t.meta[2].base, ii, jj, kk, ts, rows, limit,
-                         unit, sh_rank, tag, count);
+                         unit, sh_rank, tag);
 }
 
 // Drains a pair queue: every (i, j) against the L2 hits in the meet of both
@@ -654,8 +634,7 @@ __device__ __forceinline__ void fit_tile(const Job& j, const TV& t, int lane, co
 // timeslice 0.946 -> 0.913 ms.)
 template <bool EMIT, class TV>
 __device__ void drain(const Job& j, const TV& t, const uint32_t* queue, int lane, const Cuts& c, int qn,
-                      TSink& ts, int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag, int& count,
-                      Pending& pd) {
+                      TSink& ts, int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag, Pending& pd) {
     const float B02 = layer_pair_bound(t, 0, 2, c.K), B12 = layer_pair_bound(t, 1, 2, c.K);
     const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll 1
@@ -685,7 +664,7 @@ __device__ void drain(const Job& j, const TV& t, const uint32_t* queue, int lane
                 __syncwarp();
                 const uint32_t pe = pd.pair[lane];
                 fit_tile<EMIT>(j, t, lane, c, true, (int)(pe & 0xffffu), (int)(pe >> 16), pd.k[lane], ts, rows, limit,
-                               unit, sh_rank, tag, count);
+                               unit, sh_rank, tag);
                 __syncwarp();
                 if (cand && at >= 32) {
                     pd.pair[at - 32] = en;
@@ -701,12 +680,11 @@ __device__ void drain(const Job& j, const TV& t, const uint32_t* queue, int lane
 // The pending triples of a block-path warp, at the end of its station.
 template <bool EMIT, class TV>
 __device__ __forceinline__ void flush_pending(const Job& j, const TV& t, int lane, const Cuts& c, TSink& ts,
-                                              int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag,
-                                              int& count, Pending& pd) {
+                                              int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag, Pending& pd) {
     if (pd.m > 0) {
         const uint32_t pe = pd.pair[min(lane, pd.m - 1)];
         fit_tile<EMIT>(j, t, lane, c, lane < pd.m, (int)(pe & 0xffffu), (int)(pe >> 16), pd.k[min(lane, pd.m - 1)], ts,
-                       rows, limit, unit, sh_rank, tag, count);
+                       rows, limit, unit, sh_rank, tag);
     }
     pd.m = 0;
 }
@@ -729,15 +707,15 @@ struct RoadItems {
 // block share.  Each lane walks its own hit's L1 window.  Pairs that may belong to
 // a passing triplet are queued and drained against L2.
 template <bool EMIT, class TV>
-__device__ int enum_station(const Job& j, const TV& t, uint32_t* queue, Pending pd, int lane, const Cuts& c,
+__device__ void enum_station(const Job& j, const TV& t, uint32_t* queue, Pending pd, int lane, const Cuts& c,
                             TSink& ts, int32_t* rows, int limit, int64_t unit, int* sh_rank, int tag, int* sh_next,
                             const RoadItems* rd) {
     const int n0 = t.meta[0].nlive, n1 = t.meta[1].nlive, n2 = t.meta[2].nlive;
-    if (n0 == 0 || n1 == 0 || n2 == 0) return 0;
+    if (n0 == 0 || n1 == 0 || n2 == 0) return;
     const int n_rounds = (n0 + 31) >> 5;
     const int p0 = t.meta[0].pbase;
     const float B01 = layer_pair_bound(t, 0, 1, c.K);
-    int qn = 0, count = 0;
+    int qn = 0;
     // each warp takes the next round from the block-shared counter; items past
     // the rounds are trigger slopes to search for (CHAIN)
     auto next_round = [&]() {
@@ -783,41 +761,32 @@ __device__ int enum_station(const Job& j, const TV& t, uint32_t* queue, Pending 
             qn += __popc(mask);
             if (qn > kQCap - 32) {
                 __syncwarp();
-                drain<EMIT>(j, t, queue, lane, c, qn, ts, rows, limit, unit, sh_rank, tag, count, pd);
+                drain<EMIT>(j, t, queue, lane, c, qn, ts, rows, limit, unit, sh_rank, tag, pd);
                 qn = 0;
             }
         }
     }
     __syncwarp();
-    drain<EMIT>(j, t, queue, lane, c, qn, ts, rows, limit, unit, sh_rank, tag, count, pd);
-    flush_pending<EMIT>(j, t, lane, c, ts, rows, limit, unit, sh_rank, tag, count, pd);
-    return count;
+    drain<EMIT>(j, t, queue, lane, c, qn, ts, rows, limit, unit, sh_rank, tag, pd);
+    flush_pending<EMIT>(j, t, lane, c, ts, rows, limit, unit, sh_rank, tag, pd);
 }
 
 // Tile positions of a cell window, row by row: the first row's run [a, e)
 // is given; windows of more than one row continue on the next rows (each
 // row's columns [x0, x1] are one run of positions).
-template <int NX, int NY>
+template <int NX>
 struct WinIter {
     int p, end, row, y1, x0, x1;
     const uint16_t* bs;
-    __device__ __forceinline__ WinIter(int a, int e, const uint16_t* b, const Win& w) : p(a), end(e) {
-        if constexpr (NY > 1) {
-            bs = b;
-            row = w.y0;
-            y1 = w.y1;
-            x0 = w.x0;
-            x1 = w.x1;
-            settle();
-        }
+    __device__ __forceinline__ WinIter(int a, int e, const uint16_t* b, const Win& w)
+        : p(a), end(e), row(w.y0), y1(w.y1), x0(w.x0), x1(w.x1), bs(b) {
+        settle();
     }
     __device__ __forceinline__ void settle() {
-        if constexpr (NY > 1) {
-            while (p >= end && row < y1) {
-                ++row;
-                p = bs[row * NX + x0];
-                end = bs[row * NX + x1 + 1];
-            }
+        while (p >= end && row < y1) {
+            ++row;
+            p = bs[row * NX + x0];
+            end = bs[row * NX + x1 + 1];
         }
     }
     __device__ __forceinline__ bool valid() const { return p < end; }
@@ -846,21 +815,21 @@ __device__ bool road(const Job& j, const TV& t, const Cuts& c, float mx, float m
     const uint16_t *bs0 = t.bst, *bs1 = t.bst + TV::NC, *bs2 = t.bst + 2 * TV::NC;
     const int32_t base0 = t.meta[0].base, base1 = t.meta[1].base, base2 = t.meta[2].base;
     const float b0 = t.meta[0].bmax, b1 = t.meta[1].bmax, b2 = t.meta[2].bmax;
-    for (WinIter<TV::NX, TV::NY> i0(a[0], e[0], bs0, w[0]); i0.valid(); i0.next()) {
+    for (WinIter<TV::NX> i0(a[0], e[0], bs0, w[0]); i0.valid(); i0.next()) {
         const int p0 = i0.p;
         const float2 P0 = t.P[p0];
         if (!tube_ok(P0.x, P0.y, b0, mx, my)) continue;
         const int h0 = base0 + t.idx[p0];
         const float x0 = __ldg(j.x + h0), y0 = __ldg(j.y + h0), z0 = __ldg(j.z + h0);
         if (!tube_pass(x0, y0, z0, mx, my, c)) continue;
-        for (WinIter<TV::NX, TV::NY> i1(a[1], e[1], bs1, w[1]); i1.valid(); i1.next()) {
+        for (WinIter<TV::NX> i1(a[1], e[1], bs1, w[1]); i1.valid(); i1.next()) {
             const int p1 = i1.p;
             const float2 P1 = t.P[p1];
             if (!tube_ok(P1.x, P1.y, b1, mx, my)) continue;
             const int h1 = base1 + t.idx[p1];
             const float x1 = __ldg(j.x + h1), y1 = __ldg(j.y + h1), z1 = __ldg(j.z + h1);
             if (!tube_pass(x1, y1, z1, mx, my, c)) continue;
-            for (WinIter<TV::NX, TV::NY> i2(a[2], e[2], bs2, w[2]); i2.valid(); i2.next()) {
+            for (WinIter<TV::NX> i2(a[2], e[2], bs2, w[2]); i2.valid(); i2.next()) {
                 const int p2 = i2.p;
                 const float2 P2 = t.P[p2];
                 if (!tube_ok(P2.x, P2.y, b2, mx, my)) continue;
@@ -2080,7 +2049,7 @@ __device__ void heavy_event(const Job& j, HeavySmem& sm, const Cuts& c, int gi, 
     int trig_count = 0, nT = 0;
     for (int si = 0; si < nproc; ++si) {
         const int s = station_of(si, j.trig);
-        TSink ts{(chain || j.distinct) && si == 0, T, j.tlist_cap, &sm.s_nT, 0};
+        TSink ts{(chain || j.distinct) && si == 0, T, j.tlist_cap, &sm.s_nT};
         ts.ijk = ijk;
         ts.tt = tt;
         int cnt = 0;
@@ -2592,7 +2561,7 @@ __global__ void __launch_bounds__(kHThreads, 3) k_heavy_units(const __grid_const
         const int64_t e = j.hlist[gi];
         const int s = station_of((int)(k % per) + (EMIT ? 0 : 1), j.trig);
         load_event_offsets(j, sm, e);
-        TSink ts{false, nullptr, 0, nullptr, 0};
+        TSink ts{false, nullptr, 0, nullptr};
         int cnt = 0;
         heavy_unit<EMIT>(j, sm, c, gi, e, s, ts, j.tpool + hx, j.tpool_alive + hx, hy, cnt, -1,
                          kStream ? reinterpret_cast<const float2*>(j.tpool_ijk) + hx : nullptr);
@@ -2919,7 +2888,7 @@ __device__ bool plain_block_event(const Job& j, PlainSmem& ps, int64_t e) {
         for (int si = 0; si < nproc; ++si) {
             const int s = station_of(si, j.trig);
             if (j.unit_counts[e * S + s] == 0) continue;
-            TSink ts{false, nullptr, 0, nullptr, 0};
+            TSink ts{false, nullptr, 0, nullptr};
             int cnt = 0;
             heavy_unit<true>(j, sm, c, kGiPlain, e, s, ts, nullptr, nullptr, 0, cnt,
                              si + 1 < nproc ? station_of(si + 1, j.trig) : -1);
@@ -2946,7 +2915,7 @@ __device__ bool plain_block_event(const Job& j, PlainSmem& ps, int64_t e) {
         const int s = station_of(si, j.trig);
         if (tid == 0) sm.s_nT = 0;
         __syncthreads();
-        TSink ts{(chain || j.distinct) && si == 0, T, kPlainTCap, &sm.s_nT, 0};
+        TSink ts{(chain || j.distinct) && si == 0, T, kPlainTCap, &sm.s_nT};
         int cnt = 0;
         const int sn = si + 1 < nproc ? station_of(si + 1, j.trig) : -1;
         if (!heavy_unit<false>(j, sm, c, kGiPlain, e, s, ts, T, alive, si == 0 ? 0 : nT, cnt, sn, tt)) {
@@ -2976,7 +2945,7 @@ __device__ bool plain_block_event(const Job& j, PlainSmem& ps, int64_t e) {
             if constexpr (kStream) tt = reinterpret_cast<float2*>(j.tpool_ijk) + pb;
             if (tid == 0) sm.s_nT = 0;
             __syncthreads();
-            TSink ts2{true, T, nT, &sm.s_nT, 0};
+            TSink ts2{true, T, nT, &sm.s_nT};
             ts2.norec = true;
             ts2.ijk = ijk;
             ts2.tt = tt;
