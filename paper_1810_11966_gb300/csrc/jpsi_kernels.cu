@@ -1862,8 +1862,8 @@ __device__ __forceinline__ void light_event(const Job& j, WarpTile& w, int lane,
 
 // The warp path: every event of the batch (statically one warp per event, or
 // persistent warps grabbing `grab` events at a time).
-//   Bound by instruction issue (0.70 of the slots, ALU pipe the busiest) and, in
-// the loads of a station, by memory: 4 370 warp instructions per event of the
+//   Bound by instruction issue (0.73 of the slots, ALU pipe the busiest) and, in
+// the loads of a station, by memory: 4 205 warp instructions per event of the
 // 10^6-event workload, where sorting every hit into cells and walking windows of
 // them took 10 200.  10^6 events: 10.41 -> 4.61 ms (3.14 TB/s of hits, 0.47 of
 // the measured copy rate); the events of a 55 000-event log-normal timeslice that
