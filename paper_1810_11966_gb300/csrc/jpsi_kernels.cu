@@ -9,7 +9,8 @@
 //              pairs and triples of those are tested, and the survivors of an
 //              event's stations get the exact FP32 fit (P1) together.  CHAIN
 //              mode keeps the passing trigger triplets' slopes in the tile
-//              and searches the other stations for compatible triplets (P2).
+//              and holds the other stations' passing triplets against them
+//              (P2).
 //              Limits: 192 hits per layer, 384 per station, 32 passing trigger
 //              triplets.
 //   k_medium   the same sieve, with larger maps and one more pass, on 4-warp
@@ -137,11 +138,13 @@ struct WarpTile {
     int32_t sh[kStream ? 3 * kMaxStations : 1];  // and shifts (free-streaming windows)
     int32_t count[kMaxStations];          // passing triplets per station
     float2 T[SmallCfg::TCAP];             // trigger triplet slopes
+    using Slopes = uint32_t;              // one bit for each
+    Slopes partners[kMaxStations];        // those that have a compatible triplet in the station (CHAIN)
     union {
         unsigned long long Tijk[SmallCfg::TCAP];  // their packed hits (distinct_hits)
         float2 Tt[SmallCfg::TCAP];                // or their (min t, max t) (free-streaming windows)
     };
-    uint8_t alive[SmallCfg::TCAP];
+    uint8_t alive[SmallCfg::TCAP];        // in every station (distinct_hits)
     LayerMax lay[3];                      // of an uneven station
     static_assert(SmallCfg::LAYER_CAP <= 256, "8-bit indices");
 };
@@ -163,6 +166,8 @@ struct MediumTile {
     int red[WARPS][3];                          // largest |slope|, largest and smallest 1/z (bit patterns)
     int s_gi, s_flag;
     float2 T[TCAP];
+    using Slopes = unsigned long long;
+    Slopes partners[kMaxStations];
     union {
         unsigned long long Tijk[TCAP];
         float2 Tt[TCAP];
@@ -958,17 +963,15 @@ __device__ __forceinline__ float rcp_approx(float v) {
 }
 
 // What the warp knows of the station it staged: the pair bound of any two of
-// its hits, the tube bound of any of its hits, and the sieve's cells per unit
-// of slope.
+// its hits, and the sieve's cells per unit of slope.
 struct StationBounds {
-    float B, b, inv;
+    float B, inv;
 };
 
 // The bounds from the largest 1/z and |slope| of the station's hits.
 __device__ __forceinline__ StationBounds station_bounds(float rmax, float smax, float K) {
     StationBounds sb;
     sb.B = station_pair_bound(rmax, smax, K);
-    sb.b = __fadd_rn(__fadd_rn(__fmul_rn(K, rmax), __fmul_rn(2.0f * kKappa, smax)), kTau);
     sb.inv = __fmul_rn(0.998f, rcp_approx(sb.B));
     return sb;
 }
@@ -1084,11 +1087,18 @@ __device__ __forceinline__ void sieve_dilate(uint32_t* map, const uint32_t* othe
 // P1 on the warp's pending triples, 32 at a time, until at most `keep` of its np
 // are left (their number is returned), and what follows from a pass: the
 // triplet's rank in its unit (from the station's count), its row (emit pass),
-// its slopes if it is a trigger triplet and the event keeps them (`sink`), and
-// its entry in the scatter record.
+// its slopes if it is a trigger triplet and the event keeps them (`sink`), the nT
+// trigger slopes that it is compatible with (P2; nT is 0 until they are all known),
+// and its entry in the scatter record.
+//   The search finds every triplet of a station that passes P1, so the compatible
+// ones are among these, and P2 costs some 30 instructions per slope for 32 of them.
+// (A search of the station's hits for each slope, in turn, cost events with many
+// tracks more than all else: 20 000 events of 20 tracks and 5 other hits per layer
+// 600 us, 232 now (287 with one slope per lane on the cell-sorted tile); of 30
+// tracks and 60 hits 1 070, 554 (794).)
 template <bool EMIT, class W>
 __device__ __forceinline__ int light_fit(const Job& j, W& w, const uint32_t* pend, int lane, const Cuts& c, int64_t e,
-                                         bool sink, int np, int keep) {
+                                         bool sink, int nT, int np, int keep) {
     __syncwarp();
 #pragma unroll 1
     while (np > keep) {
@@ -1111,10 +1121,21 @@ __device__ __forceinline__ int light_fit(const Job& j, W& w, const uint32_t* pen
             const float ys[3] = {__ldg(j.y + h0), __ldg(j.y + h1), __ldg(j.y + h2)};
             const float zs[3] = {__ldg(j.z + h0), __ldg(j.z + h1), __ldg(j.z + h2)};
             ok = fit_pass(xs, ys, zs, c, mx, my);
-            if constexpr (kStream) {  // coincident, and owned by this window
-                ok = ok && coincident3(__ldg(j.t + h0), __ldg(j.t + h1), __ldg(j.t + h2), j.dt, tt.x, tt.y) &&
-                     tt.x >= __ldg(j.wb + e) && tt.x < __ldg(j.wb + e + 1);
+            if constexpr (kStream)
+                ok = ok && coincident3(__ldg(j.t + h0), __ldg(j.t + h1), __ldg(j.t + h2), j.dt, tt.x, tt.y);
+            if (!EMIT && ok) {
+                typename W::Slopes with = 0;
+#pragma unroll 1
+                for (int ti = 0; ti < nT; ++ti) {
+                    const float2 m = w.T[ti];
+                    if (chain_pass(xs, ys, zs, m.x, m.y, c) &&
+                        (!kStream || partner_coincident(tt.x, tt.y, w.Tt[ti], j.dt)))
+                        with |= (typename W::Slopes)1 << ti;
+                }
+                if (with) atomicOr(&w.partners[st], with);
             }
+            // (free-streaming windows: a triplet counts where it is owned, a partner anywhere)
+            if constexpr (kStream) ok = ok && tt.x >= __ldg(j.wb + e) && tt.x < __ldg(j.wb + e + 1);
         }
         int rank = 0;
         if (ok) {
@@ -1503,7 +1524,7 @@ template <bool EMIT, bool FILTER, class W, class R, class L>
 __device__ __forceinline__ void sieve_triples(const Job& j, W& w, uint32_t* pend, int lane, const Cuts& c, float B,
                                               int64_t e, int s, int s1, int s2, const L* l0, int m0, const L* l1,
                                               int m1, const L* l2, int m2, int k_first, int k_step, bool sink,
-                                              bool all, bool crowded, R& rows, int& np) {
+                                              int nT, bool all, bool crowded, R& rows, int& np) {
     const uint32_t lt = (1u << lane) - 1u;
     const int hi0 = l0[min(lane, max(m0 - 1, 0))];  // what is left of layer 0, its first 32
     const float2 Pi0 = w.P[m0 > 0 ? hi0 : 0];
@@ -1569,7 +1590,7 @@ __device__ __forceinline__ void sieve_triples(const Job& j, W& w, uint32_t* pend
             }
         }
         np = uniform(np);
-        np = light_fit<EMIT>(j, w, pend, lane, c, e, sink, np, all && !more ? 0 : 32);
+        np = light_fit<EMIT>(j, w, pend, lane, c, e, sink, nT, np, all && !more ? 0 : 32);
         if (!more) break;
     }
 }
@@ -1588,8 +1609,7 @@ constexpr int kCrowdedWarp = 12, kCrowdedBlock = 24;
 // a hit with z <= 0 or 2 for one whose pruning bound is not finite.
 template <bool EMIT>
 __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane, const Cuts& c, int32_t o0, int n0,
-                                             int n1, int n2, int64_t e, int s, bool sink, bool all, StationBounds& sb,
-                                             int& np) {
+                                             int n1, int n2, int64_t e, int s, bool sink, int nT, bool all, int& np) {
     const int most = max(max(n0, n1), n2);
     const Shift3 sh = kStream ? Shift3{uniform(w.sh[3 * s]), uniform(w.sh[3 * s + 1]), uniform(w.sh[3 * s + 2])}
                               : Shift3{0, 0, 0};
@@ -1601,7 +1621,7 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
         ok = sieve_stage<4>(j, w, lane, o0, n0, n1, n2, sh, rmax, smax);
     else
         ok = sieve_stage<6>(j, w, lane, o0, n0, n1, n2, sh, rmax, smax);
-    sb = station_bounds(rmax, smax, j.K);
+    StationBounds sb = station_bounds(rmax, smax, j.K);
     if (__builtin_expect(!uniform(ok && sb.B < INFINITY), 0)) {
         const int st = uniform(sieve_classify(j, w.P, lane, o0, n0, n0 + n1, n0 + n1 + n2, sh, w.lay, rmax, smax));
         if (st) return st;
@@ -1627,62 +1647,8 @@ __device__ __forceinline__ int light_station(const Job& j, WarpTile& w, int lane
                       m0, -1, n1, SmallCfg::LAYER_CAP, m2, n0, n0 + n1);
     if (m2 > 0 || (all && np > 0))
         sieve_triples<EMIT, false>(j, w, w.pend, lane, c, sb.B, e, s, n0, n0 + n1, w.left[0], m0,
-                                   (const uint8_t*)nullptr, n1, w.left[1], m2, 0, 1, sink, all, crowded, rows, np);
+                                   (const uint8_t*)nullptr, n1, w.left[1], m2, 0, 1, sink, nT, all, crowded, rows, np);
     return 0;
-}
-
-// Does the staged station hold a passing triplet compatible with the trigger
-// slopes (mx, my)?  The warp tests the tube on 32 hits a step; every hit of
-// layer 0 that passes it is tried with every such hit of layer 1, and those
-// pairs with 32 hits of layer 2 a step (P1 and P2).  Warp-uniform.
-template <class W>
-__device__ bool sieve_road(const Job& j, const W& w, int lane, const Cuts& c, const StationBounds& sb,
-                           int32_t o0, int n0, int n1, int n2, const Shift3& sh, float mx, float my, float2 Tt) {
-    const int s1 = n0, s2 = n0 + n1, n = s2 + n2;
-    // the hits of places [p0, p0 + 32) of a layer ending at `end` (hit index less place: g) that pass the tube
-    auto tube = [&](int p0, int end, int32_t g) {
-        bool in = false;
-        const float2 s = w.P[p0 + lane];
-        if (p0 + lane < end && tube_ok(s.x, s.y, sb.b, mx, my)) {
-            const int32_t h = g + p0 + lane;
-            in = tube_pass(__ldg(j.x + h), __ldg(j.y + h), __ldg(j.z + h), mx, my, c);
-        }
-        return (unsigned)uniform((int)__ballot_sync(kFull, in));
-    };
-#pragma unroll 1
-    for (int i0 = 0; i0 < n0; i0 += 32) {
-#pragma unroll 1
-        for (unsigned mi = tube(i0, s1, o0 + sh.a); mi; mi &= mi - 1) {
-            const int32_t h0 = o0 + sh.a + i0 + __ffs(mi) - 1;
-#pragma unroll 1
-            for (int j0 = s1; j0 < s2; j0 += 32) {
-#pragma unroll 1
-                for (unsigned mj = tube(j0, s2, o0 + sh.b); mj; mj &= mj - 1) {
-                    const int32_t h1 = o0 + sh.b + j0 + __ffs(mj) - 1;
-#pragma unroll 1
-                    for (int k0 = s2; k0 < n; k0 += 32) {
-                        const float2 s = w.P[k0 + lane];
-                        bool ok = false;
-                        if (k0 + lane < n && tube_ok(s.x, s.y, sb.b, mx, my)) {
-                            const int32_t h2 = o0 + sh.c + k0 + lane;
-                            const float xs[3] = {__ldg(j.x + h0), __ldg(j.x + h1), __ldg(j.x + h2)};
-                            const float ys[3] = {__ldg(j.y + h0), __ldg(j.y + h1), __ldg(j.y + h2)};
-                            const float zs[3] = {__ldg(j.z + h0), __ldg(j.z + h1), __ldg(j.z + h2)};
-                            float fx, fy;
-                            ok = chain_pass(xs, ys, zs, mx, my, c) && fit_pass(xs, ys, zs, c, fx, fy);
-                            if constexpr (kStream) {
-                                float pmin, pmax;
-                                coincident3(__ldg(j.t + h0), __ldg(j.t + h1), __ldg(j.t + h2), j.dt, pmin, pmax);
-                                ok = ok && partner_coincident(pmin, pmax, Tt, j.dt);
-                            }
-                        }
-                        if (uniform(__any_sync(kFull, ok))) return true;
-                    }
-                }
-            }
-        }
-    }
-    return false;
 }
 
 __device__ __forceinline__ void push_event(const Job& j, int64_t e, uint8_t cls) {
@@ -1767,7 +1733,10 @@ __device__ void light_event_count(const Job& j, WarpTile& w, int lane, const Cut
             prefetch_hits_l2(j, o0, w.off[3 * j.trig + 3], lane);
         const bool sink = chain || j.distinct;  // the trigger triplets are kept: CHAIN slopes, candidates' hits
         int np = 0, nT = 0;
-        if (lane < kMaxStations) w.count[lane] = 0;
+        if (lane < kMaxStations) {
+            w.count[lane] = 0;
+            w.partners[lane] = 0;
+        }
 #pragma unroll 1
         for (int si = 0; si < nproc; ++si) {
             const int s = station_of(si, j.trig);
@@ -1775,9 +1744,8 @@ __device__ void light_event_count(const Job& j, WarpTile& w, int lane, const Cut
             const int n0 = uniform(w.off[3 * s + 1]) - o0, n1 = uniform(w.off[3 * s + 2]) - o0 - n0,
                       n2 = uniform(w.off[3 * s + 3]) - o0 - n0 - n1;
             if (si + 1 < nproc) prefetch_station(j, w.off, w.sh, station_of(si + 1, j.trig), lane);
-            StationBounds sb;
-            const int st = light_station<false>(j, w, lane, c, o0, n0, n1, n2, e, s, sink,
-                                                (sink && si == 0) || si + 1 == nproc, sb, np);
+            const int st = light_station<false>(j, w, lane, c, o0, n0, n1, n2, e, s, sink, chain ? nT : 0,
+                                                (sink && si == 0) || si + 1 == nproc, np);
             if (st != 0) {
                 moved = st == 1 ? kClsInvalid : kClsGeneric;
                 break;
@@ -1788,16 +1756,6 @@ __device__ void light_event_count(const Job& j, WarpTile& w, int lane, const Cut
                     moved = kClsHeavy;
                     break;
                 }
-                if (lane < nT) w.alive[lane] = 1;  // (at most 32)
-            } else {
-#pragma unroll 1
-                for (int ti = 0; ti < nT; ++ti) {  // (CHAIN only: PAPER has one station)
-                    if (!uniform(w.alive[ti])) continue;  // (uniform: see RowLists)
-                    const float2 m = w.T[ti];
-                    const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, shift3(w.sh, s), m.x, m.y,
-                                                  kStream ? w.Tt[ti] : make_float2(0.f, 0.f));
-                    if (!found && lane == 0) w.alive[ti] = 0;
-                }
             }
             __syncwarp();  // the tile may be staged again
         }
@@ -1805,7 +1763,13 @@ __device__ void light_event_count(const Job& j, WarpTile& w, int lane, const Cut
             static_assert(SmallCfg::TCAP <= 32, "one flag per lane");
             if (lane < S) j.unit_counts[e * S + lane] = w.count[lane];
             int tc = w.count[j.trig];
-            if (chain) tc = __popc(__ballot_sync(kFull, lane < nT && w.alive[lane]));
+            if (chain) {  // the slopes with a partner in every other station
+                const unsigned with = __reduce_and_sync(
+                    kFull, lane < S && lane != j.trig ? w.partners[lane] : nT < 32 ? (1u << nT) - 1u : ~0u);
+                tc = __popc(with);
+                w.alive[lane] = with >> lane & 1u;
+                __syncwarp();
+            }
             if (j.distinct) {  // nT is warp-uniform
                 const bool f = nT >= 2 && warp_disjoint_pair(w.Tijk, chain ? w.alive : nullptr, nT, lane);
                 if (lane == 0) j.dpair[e] = f;
@@ -1845,8 +1809,7 @@ __device__ void light_event_emit(const Job& j, WarpTile& w, int lane, const Cuts
         const int32_t o0 = uniform(w.off[3 * s]);
         const int n0 = uniform(w.off[3 * s + 1]) - o0, n1 = uniform(w.off[3 * s + 2]) - o0 - n0,
                   n2 = uniform(w.off[3 * s + 3]) - o0 - n0 - n1;
-        StationBounds sb;
-        const int st = light_station<true>(j, w, lane, c, o0, n0, n1, n2, e, s, false, true, sb, np);
+        const int st = light_station<true>(j, w, lane, c, o0, n0, n1, n2, e, s, false, 0, true, np);
         if ((st != 0 || w.count[s] != cnt) && lane == 0) atomicOr(&j.ctrl->status, kStEmitMismatch);
         __syncwarp();
     }
@@ -2114,11 +2077,11 @@ __device__ void heavy_event(const Job& j, HeavySmem& sm, const Cuts& c, int gi, 
 // Medium path: 4-warp blocks take the events of the medium list, one at a time, and
 // run every station of their event with the sieve of the warp path, shared by the
 // warps: the trigger station first (in CHAIN mode its passing triplets'
-// slopes, at most kTCap, stay in shared memory), then the others and the searches
-// for those slopes.  An event with more trigger slopes goes on to the block tile;
-// one with extreme coordinates to the unpruned kernel.
+// slopes, at most kTCap, stay in shared memory), then the others, whose passing
+// triplets are held against those slopes.  An event with more trigger slopes goes on
+// to the block tile; one with extreme coordinates to the unpruned kernel.
 //   Bound by instruction issue and the barriers between the maps.  The events of
-// a 55 000-event log-normal timeslice: 379 us with cell-sorted tiles, 280 with
+// a 55 000-event log-normal timeslice: 379 us with cell-sorted tiles, 260 with
 // the sieve; of 100 000 free-streaming collisions: 1.23 -> 1.02 ms.  Four warps and
 // eight blocks per SM (64 registers) against two warps and 13 blocks: the same
 // on the timeslice, 4 % slower on the collisions, but an event takes little more than
@@ -2201,7 +2164,7 @@ __device__ __forceinline__ void medium_pass(const Job& j, MediumTile& w, float i
 constexpr int kFilterMin = 8;
 template <bool EMIT>
 __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const Cuts& c, int64_t e, int s, bool sink,
-                                              bool all, StationBounds& sb, int& np) {
+                                              int nT, bool all, int& np) {
     const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
     const int32_t o0 = uniform(w.off[3 * s]);
     const int n0 = uniform(w.off[3 * s + 1]) - o0, n1 = uniform(w.off[3 * s + 2]) - o0 - n0,
@@ -2210,6 +2173,7 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
     constexpr int T = MediumTile::THREADS;
     const Shift3 sh = shift3(w.sh, s);
     float smax = 0.0f, rmax = 0.0f, rmin = INFINITY;
+    StationBounds sb;
     for (int p0 = 0; p0 < n; p0 += 4 * T) {
         float x[4], y[4], z[4];
 #pragma unroll
@@ -2318,7 +2282,7 @@ __device__ __forceinline__ int medium_station(const Job& j, MediumTile& w, const
         row_lists<T>(j, rows, w.P, tid, uneven ? pair_bounds(w.lay, j.K) : PairBounds{sb.B, sb.B, sb.B}, w.left[0], m0,
                      l1 ? MediumCfg::LAYER_CAP : -1, m1, 2 * MediumCfg::LAYER_CAP, m2, s1, s2);
     sieve_triples<EMIT, true>(j, w, w.pend[wp], lane, c, sb.B, e, s, s1, s2, w.left[0], m0, l1, m1, w.left[2], m2, wp,
-                              MediumTile::WARPS, sink, all, crowded, rows, np);
+                              MediumTile::WARPS, sink, nT, all, crowded, rows, np);
     return 0;
 }
 
@@ -2332,7 +2296,10 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
         w.off[i] = __ldg(j.off + e * 3 * S + i);
         if (kStream && i < 3 * S) w.sh[i] = __ldg(j.shift + e * 3 * S + i);
     }
-    if (tid < kMaxStations) w.count[tid] = 0;
+    if (tid < kMaxStations) {
+        w.count[tid] = 0;
+        w.partners[tid] = 0;
+    }
     __syncthreads();
     int np = 0, nT = 0;
     const bool sink = !EMIT && (chain || j.distinct);
@@ -2345,8 +2312,8 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
             if (si == 0) prefetch_station(j, w.off, w.sh, s, lane);
             if (si + 1 < nproc) prefetch_station(j, w.off, w.sh, station_of(si + 1, j.trig), lane);
         }
-        StationBounds sb;
-        const int st = medium_station<EMIT>(j, w, c, e, s, sink, EMIT || (sink && si == 0) || si + 1 == nproc, sb, np);
+        const int st = medium_station<EMIT>(j, w, c, e, s, sink, chain ? nT : 0,
+                                            EMIT || (sink && si == 0) || si + 1 == nproc, np);
         if (EMIT) {
             __syncthreads();
             if ((st != 0 || w.count[s] != cnt) && tid == 0) atomicOr(&j.ctrl->status, kStEmitMismatch);
@@ -2370,19 +2337,6 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
                 if (tid == 0) push_event(j, e, kClsHeavy);
                 return;
             }
-            if (tid < nT) w.alive[tid] = 1;
-        } else {
-            const int32_t o0 = w.off[3 * s];
-            const int n0 = w.off[3 * s + 1] - o0, n1 = w.off[3 * s + 2] - o0 - n0, n2 = w.off[3 * s + 3] - o0 - n0 - n1;
-#pragma unroll 1
-            for (int ti = wp; ti < nT; ti += MediumTile::WARPS) {  // (CHAIN only: PAPER has one station)
-                if (!uniform(w.alive[ti])) continue;  // (uniform: see RowLists)
-                const float2 m = w.T[ti];
-                const bool found = sieve_road(j, w, lane, c, sb, o0, n0, n1, n2, shift3(w.sh, s), m.x, m.y,
-                                              kStream ? w.Tt[ti] : make_float2(0.f, 0.f));
-                __syncwarp();
-                if (!found && lane == 0) w.alive[ti] = 0;
-            }
         }
         __syncthreads();  // the tile may be staged again
     }
@@ -2390,7 +2344,12 @@ __device__ void medium_event(const Job& j, MediumTile& w, const Cuts& c, int64_t
     static_assert(kTCap <= MediumTile::THREADS, "one flag per thread");
     if (tid < S) j.unit_counts[e * S + tid] = w.count[tid];
     int tc = w.count[j.trig];
-    if (chain) tc = __syncthreads_count(tid < nT && w.alive[tid]);
+    if (chain) {  // the slopes with a partner in every other station
+        bool with = tid < nT;
+        for (int s = 0; s < S; ++s) with = with && (s == j.trig || (w.partners[s] >> tid & 1ull));
+        if (tid < MediumTile::TCAP) w.alive[tid] = with;
+        tc = __syncthreads_count(with);
+    }
     if (j.distinct) {
         const bool f =
             nT >= 2 && block_disjoint_pair<MediumTile::THREADS>(w.Tijk, chain ? w.alive : nullptr, nT, &w.s_flag);

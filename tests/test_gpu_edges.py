@@ -397,3 +397,47 @@ def test_z_table_of_many_stations(lib, oracle_mod, S, host):
         tracks = dt.cpu().numpy()
     assert np.array_equal(tracks, ref["track_counts"]) and o.trip_needed == ref["trip_needed"]
     ctx.close()
+
+
+def _track_events(rng, counts, S, n_other, missing=()):
+    """Events of straight tracks (counts: how many in each) and n_other hits per layer; every third track
+    has no hits in the stations of `missing`."""
+    events = []
+    for n in counts:
+        # far enough apart that their hits make no triplets of mixed tracks
+        g = int(np.ceil(np.sqrt(max(n, 1))))
+        grid = [(0.6 * (k % g + 0.5) / g - 0.3, 0.6 * (k // g + 0.5) / g - 0.3) for k in range(n)]
+        ev = []
+        for q, z in enumerate(layer_z(S)):
+            hits = [(tx * z + rng.normal(0, 0.02), ty * z + rng.normal(0, 0.02), z) for k, (tx, ty) in enumerate(grid)
+                    if not (q // 3 in missing and k % 3 == 0)]
+            r, phi = rng.uniform(0.5, 0.6, n_other) * z, rng.uniform(0, 2 * np.pi, n_other)
+            hits += [(a * np.cos(p), a * np.sin(p), z) for a, p in zip(r, phi)]
+            rng.shuffle(hits)
+            ev.append(hits)
+        events.append(ev)
+    return make_batch(events, S)
+
+
+@pytest.mark.parametrize("n_other", [0, 150, 200])
+@pytest.mark.parametrize("missing", [(), (0,), (0, 1)])
+def test_trigger_slopes_up_to_the_paths_limits(lib, oracle_mod, n_other, missing):
+    # 32 trigger triplets on a warp, 64 on a medium block, and one more or less; all or
+    # some of them without a partner in one or two stations
+    rng = np.random.default_rng(300 + n_other + len(missing))
+    b = _track_events(rng, [0, 1, 2, 31, 32, 33, 63, 64, 65], 3, n_other, missing)
+    ref = oracle_mod.run(oracle_mod.params(3, 1, t_xz=0.04), b)
+    assert ref["track_counts"].max() >= (65 if not missing else 40)
+    _oracle_same(lib, oracle_mod, b, 3, 0.04, modes=(1,), record_caps=(-1, 0), label=f"{n_other} {missing}")
+
+
+def test_many_tracks_keep_their_speed(lib):
+    # 20 tracks and 5 other hits per layer against 25 hits without tracks: 1.6 times
+    # the time.  Searching every station for one trigger slope after the other took 5.
+    rng = np.random.default_rng(21)
+    tracks = _track_events(rng, [20] * 400, 4, 5)
+    n = 50  # 400 different events, 50 times over
+    tracks = {**{k: np.tile(tracks[k], n) for k in ("x", "y", "z")}, "n_events": 400 * n, "n_hits": tracks["n_hits"] * n,
+              "offsets": np.arange(400 * n * 12 + 1, dtype=np.int32) * 25, "n_stations": 4}
+    t = [_time_us(_selection(lib, b, 4, 1, 0.5)) for b in (_random_batch(400 * n, 4, 25, 22), tracks)]
+    assert t[1] < 3.0 * t[0], t
