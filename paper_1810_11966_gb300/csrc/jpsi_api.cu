@@ -413,12 +413,14 @@ jpsi_status state_init(jpsi_ctx* c, RunState& rs) {
     return JPSI_OK;
 }
 
+void destroy_graph(Graph& g) {
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    if (g.g) cudaGraphDestroy(g.g);
+    g = Graph{};
+}
+
 void destroy_graphs(RunState& rs) {
-    for (Graph& g : rs.graphs) {
-        if (g.exec) cudaGraphExecDestroy(g.exec);
-        if (g.g) cudaGraphDestroy(g.g);
-        g = Graph{};
-    }
+    for (Graph& g : rs.graphs) destroy_graph(g);
 }
 
 void state_free(jpsi_ctx* c, RunState& rs) {
@@ -466,6 +468,7 @@ jpsi_status phase_graph(jpsi_ctx* c, RunState& rs, Phase phase, const Launchers&
     if (G.exec && same) return JPSI_OK;
     std::lock_guard<std::mutex> cap_lock(c->cap_mu);
     if (!same) destroy_graphs(rs);
+    destroy_graph(G);  // (what a failed capture left)
     rs.g_cfg_id = c->cfg_id;
     rs.g_stream = L.stream;
     cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
@@ -485,8 +488,6 @@ jpsi_status phase_graph(jpsi_ctx* c, RunState& rs, Phase phase, const Launchers&
     if ((e = cudaGraphGetNodes(G.g, nullptr, &n)) != cudaSuccess) return cuda_fail(c, e, "graph nodes");
     std::vector<cudaGraphNode_t> all(n);
     if (n && (e = cudaGraphGetNodes(G.g, all.data(), &n)) != cudaSuccess) return cuda_fail(c, e, "graph nodes");
-    G.nodes.clear();
-    G.params.clear();
     for (cudaGraphNode_t node : all) {
         cudaGraphNodeType t;
         if ((e = cudaGraphNodeGetType(node, &t)) != cudaSuccess) return cuda_fail(c, e, "graph node type");
