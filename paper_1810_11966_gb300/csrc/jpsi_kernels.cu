@@ -1825,12 +1825,12 @@ __device__ __forceinline__ void light_event(const Job& j, WarpTile& w, int lane,
 
 // The warp path: every event of the batch (statically one warp per event, or
 // persistent warps grabbing `grab` events at a time).
-//   Bound by instruction issue (0.73 of the slots, ALU pipe the busiest) and, in
-// the loads of a station, by memory: 4 205 warp instructions per event of the
+//   Bound by instruction issue (0.75 of the slots, ALU pipe the busiest) and, in
+// the loads of a station, by memory: 4 045 warp instructions per event of the
 // 10^6-event workload, where sorting every hit into cells and walking windows of
-// them took 10 200.  10^6 events: 10.41 -> 4.61 ms (3.14 TB/s of hits, 0.47 of
+// them took 10 200.  10^6 events: 10.41 -> 4.30 ms (3.37 TB/s of hits, 0.50 of
 // the measured copy rate); the events of a 55 000-event log-normal timeslice that
-// fit: 0.394 -> 0.208 ms; 80 000 events in PAPER mode: 0.212 -> 0.105 ms.
+// fit: 0.394 -> 0.190 ms; 80 000 events in PAPER mode: 0.212 -> 0.102 ms.
 //   72 registers (28 warps per SM) were measured before the row lists: 4.73 ms,
 // against 4.86 with 64 (32 warps, a few spills) and 80 (24 warps) and 5.40 with 56.
 template <bool EMIT>
