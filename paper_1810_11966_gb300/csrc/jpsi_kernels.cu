@@ -1596,13 +1596,14 @@ __device__ __forceinline__ void sieve_triples(const Job& j, W& w, uint32_t* pend
 }
 
 // Hits left of layer 2 beyond which a station is crowded: where the row lists cost
-// less than trying each of those hits with all of layer 1.  One warp, limits 8, 12
-// and 18: 20 000 events of 100 hits per layer with a 1 cm window 515, 526 and 555 us
-// (639 without row lists), 10^6 events with 0.5 cm, where few stations have as
-// many, 5.43, 5.33 and 5.33 ms.  A block shares those hits between four warps: 12, 16
-// and 24 differ by less than 3 %.  Row lists made events of 250 hits per layer with
-// a 1 cm window (medium path, 3 000 events) 376 us, 599 on the block tile and 818
-// without them; 200 hits 297, 554; 100 hits with 2 cm (warp path) 592, 1 401.
+// less than trying each of those hits with all of layer 1.  One warp, limits 8, 12,
+// 18 and 24: 40 000 events of 50 hits per layer with a 2 cm window 464, 471, 503 and
+// 554 us, of 100 hits with 1 cm 441, 444, 466 and 507; the other way about, 60 hits
+// with 1 cm (noalloc) 178, 172, 167 and 166, 100 hits with 0.7 cm 341, 325, 330 and
+// 332.  A block shares those hits between four warps; limits 12, 24, 48 and 80: 150
+// hits with 0.7 cm 223, 219, 221 and 223, with 1 cm 277, 280, 305 and 357; 250 hits with
+// 0.7 cm 219, 217, 240 and 292.  Row lists made events of 250 hits per layer with a
+// 1 cm window (3 000 events) 387 us, 599 on the block tile and 818 without them.
 constexpr int kCrowdedWarp = 12, kCrowdedBlock = 24;
 
 // Stages station s of event e and finds its triples (see above).  Returns 0, 1 for
